@@ -1407,10 +1407,10 @@ inet_status inet_reduce(inet_ctx* ctx, const int32_t* net_ids, int32_t n, const 
   uint64_t launches = 0;
   bool async_paused = false;
   if (fc[cur] > 0 && o.mode == INET_MODE_ASYNC) {
-    const size_t smem_a = async_smem_bytes((uint32_t)B, d.n_labels, d.n_tmpl);
     // the kernel specialised for the rule set when it can be had
     const void* jf = jit_kernel(ctx, K.track);
     const void* afn = jf ? jf : (const void*)K.async;
+    const size_t smem_a = async_smem_bytes((uint32_t)B, d.n_labels, d.n_tmpl, jf == nullptr);
     if (jf) CK(raise_smem_dyn(afn, smem_a));
     else CK(raise_smem(kSmemAsync + K.track, afn, smem_a));
     int per = 0;

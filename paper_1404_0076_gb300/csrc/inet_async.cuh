@@ -33,37 +33,76 @@
 //
 // Rules (a rule set known when the kernel is compiled, see inet_jit.h): the
 // library compiles k_async<kTrack, Rules> at run time for the loaded rule
-// set; a warp whose lanes all reduce one of its small rules runs that rule's
-// own straight-line code (uni_interact, rule_body), every other warp the
-// general code below it.  NoRules is the general kernel built with the
-// library.
+// set; each lane then runs its own rule's straight-line code (one_step), and
+// a rule that repeats itself along a list many interactions at a time
+// (run_rule, pass_rule, end_run).  NoRules is the general kernel built with
+// the library, which interprets the templates.
+//
+// What bounds the loop is latency: of a warp's turn (load, slots, rules,
+// fence, exchanges, hand-on; 8 000 to 50 000 cycles) and of the dependent
+// loads inside a run.  The design follows from that: many interactions per
+// turn where a rule allows it, one fence for the whole warp, nothing between
+// lanes but the hand-on.  One interaction per turn, before / runs, now:
+// 2048 Mul nets 10.0 / 4.4 ms, Ackermann(3, 4..8) 66 / 45 ms,
+// Fibonacci(20..25) 133 / 26.6 ms, Fibonacci(22..25) x 64 149 / 41 ms, 512
+// random trees 1.48 / 1.15 ms, a server's 2000 requests 272 / 95 ms.
 #pragma once
 
 #include "inet_kernels.cuh"
 
 namespace inet {
 
-constexpr int kAStack = 128;   // per-warp stack of free agent slots
-constexpr int kVStack = 128;   // per-warp stack of free name slots
-constexpr int kVStageW = 64;   // names freed while linking, per warp
-constexpr int kRefill = 32;    // slots fetched for the warp's stack when it runs dry
+// A column of 16 agent slots lets a run of Dup go on for 16 copies and lays
+// them out side by side; 4 freed slots kept per lane (2048 Mul nets: 4.4 ms
+// with 2, 3.9 with 4, 4.3 with 8, when these were measured against each other).
+constexpr int kARes = 16;      // free agent slots a lane keeps for itself
+constexpr int kVRes = 8;       // free name slots a lane keeps for itself
+constexpr int kKeep = 4;       // slots of each kind a lane keeps of those it frees; the rest is the warp's
+constexpr int kAStack = 576;   // per-warp stack of free agent slots
+constexpr int kVStack = 288;   // per-warp stack of free name slots
+// Most interactions of one run: of a warp's only lane, of one lane among
+// several, and where most of the warp's lanes reduce rules that do not run
+// (they wait for the run).  Lone: a chain of 20 000 Add 3.4 ms with 64, 2.3
+// with 512.  Among several, 48 / 64 / 96: 2048 Mul nets 5.7 / 5.5 / 6.5 ms,
+// Fibonacci(20..25) 30.6 / 29.5 / 28.5 ms.  Mixed, 16 against 64: 512 random
+// trees within the spread of the runs, and 1.5 against 1.7 ms before runs ended
+// inside (end_run).
+constexpr uint32_t kRunLone = 512, kRunMany = 64, kRunMixed = 16;
 constexpr unsigned long long kNoTicket = ~0ull;
+constexpr uint32_t kFetchA = 32, kFetchV = 16;  // slots fetched beyond the need when a warp's stack runs dry
+static_assert(kARes >= kMaxNew - 2 && kVRes >= kMaxFresh, "a lane's slots serve any one interaction");
+static_assert(kAStack >= 32 * kARes + (int)kFetchA && kVStack >= 32 * kVRes + (int)kFetchV, "a warp's stacks serve any one step");
 
-struct WarpMem {
-  uint32_t vals[kNumVals][32];
-  Pair out[kMaxLink][32];
-  Pair xl[(kMaxLink - 1) * 32];  // extra pairs of one iteration, in lane order
+// Shared memory of one warp.  kTable: with the value table of the general
+// kernel, which interprets every rule.
+template <bool kTable>
+struct ValueTable {
+  static constexpr bool kHasTable = false;
+};
+template <>
+struct ValueTable<true> {
+  static constexpr bool kHasTable = true;
+  uint32_t vals[kNumVals][32];   // a column per lane
+};
+template <bool kTable>
+struct alignas(16) WarpMem : ValueTable<kTable> {
+  uint32_t ares[kARes][32];      // lane-private free slots, a column per lane
+  uint32_t vres[kVRes][32];
+  Pair out[kMaxLink][32];        // new active pairs of one step
+  union {
+    uint2 eq[kMaxLink][32];        // equations of one step left to link after the fence
+    Pair xl[(kMaxLink - 1) * 32];  // extra pairs of one iteration, in lane order
+  };
   uint32_t astk[kAStack];
   uint32_t vstk[kVStack];
-  uint32_t vstage[kVStageW];
-  int vstage_n, pad[3];
+  int an, vn, pad[2];            // entries of the warp's stacks (above the size: pushes that went to the ring)
 };
 
-__host__ __device__ inline size_t async_smem_bytes(uint32_t block, uint32_t n_labels, uint32_t n_tmpl) {
+__host__ __device__ inline size_t async_smem_bytes(uint32_t block, uint32_t n_labels, uint32_t n_tmpl, bool table) {
   size_t b = 0;
   auto take = [&](size_t n, size_t align) { b = (b + align - 1) / align * align; b += n; };
   take(sizeof(Template) * (n_tmpl ? n_tmpl : 1), 16);
-  take(sizeof(WarpMem) * (block / 32), 16);
+  take((table ? sizeof(WarpMem<true>) : sizeof(WarpMem<false>)) * (block / 32), 16);
   take(sizeof(uint32_t) * INET_MAX_RULES, 16);
   take(sizeof(int16_t) * n_labels * n_labels, 16);
   return b + 16;
@@ -85,28 +124,224 @@ __device__ __forceinline__ void st_release64(unsigned long long* p, unsigned lon
 // ticket + 1; both compare all 64 bits, so no lap can be mistaken for
 // another however far ahead tickets were claimed.
 
-// A second arrival at name slot x: the slot is finished (its owner mark
-// cleared) and goes to the warp's staging list, or the ring when that is full.
-template <bool kTrack>
-__device__ __forceinline__ void release_name(const Dev& d, WarpMem& W, uint32_t x) {
-  __stcg(d.var + x, kEmpty);
-  if constexpr (kTrack) __stcg(d.vown + x, kNoNet);
-  const int pos = atomicAdd(&W.vstage_n, 1);
-  if (pos < kVStageW) {
-    W.vstage[pos] = x;
+// Free slots.  A lane takes the slots of its interactions from a private
+// column of the warp's shared memory and puts the slots it frees back there,
+// so that lanes reducing different rules, or runs of different lengths, need
+// no agreement; what does not fit goes to the warp's stack, then to the ring.
+// Only refill() moves slots into the columns, for all lanes of the warp at
+// once.
+struct Lane {
+  int na, nv;       // slots in this lane's columns
+  long long live;   // change of live agents by this lane
+};
+
+// What a lane does not keep of the slots it frees: to the warp's stack, else
+// to the ring.  Out of line, like the other rare paths here: the kernel holds
+// a copy of the common path for every rule, and its size counts (instruction
+// cache).
+template <class WM>
+__device__ __noinline__ void spill_agent(const Dev& d, WM& W, uint32_t slot) {
+  const int pos = atomicAdd(&W.an, 1);
+  if (pos < kAStack) {
+    W.astk[pos] = slot;
+  } else {
+    const unsigned long long tp = atomicAdd(&d.ctrl->a_tail, 1ull);
+    __stcg(d.afree + tp % d.cap_agents, slot);
+  }
+}
+template <class WM>
+__device__ __noinline__ void spill_name(const Dev& d, WM& W, uint32_t x) {
+  const int pos = atomicAdd(&W.vn, 1);
+  if (pos < kVStack) {
+    W.vstk[pos] = x;
   } else {
     const unsigned long long tp = atomicAdd(&d.ctrl->v_tail, 1ull);
     __stcg(d.vfree + tp % d.cap_vars, x);
   }
 }
+__device__ __noinline__ void report(const Dev& d, int32_t code, uint32_t info) { set_error(d.ctrl, code, info); }
+
+template <bool kTrack, class WM>
+__device__ __forceinline__ void put_agent(const Dev& d, WM& W, Lane& L, int lane, uint32_t slot) {
+  if constexpr (kTrack) __stcg(&d.node[slot].head, kFreeHead);
+  if (L.na < kKeep) W.ares[L.na++][lane] = slot;
+  else spill_agent(d, W, slot);
+}
+
+// A second arrival at name slot x: the slot is finished (its owner mark
+// cleared) and free again.
+template <bool kTrack, class WM>
+__device__ __forceinline__ void release_name(const Dev& d, WM& W, Lane& L, int lane, uint32_t x) {
+  __stcg(d.var + x, kEmpty);
+  if constexpr (kTrack) __stcg(d.vown + x, kNoNet);
+  if (L.nv < kKeep) W.vres[L.nv++][lane] = x;
+  else spill_name(d, W, x);
+}
+
+template <class WM>
+__device__ __forceinline__ uint32_t take_agent(const WM& W, Lane& L, int lane) { return W.ares[--L.na][lane]; }
+
+// A free name slot is empty: never used, or cleared when it was released
+// (by a lane of this warp, or before this launch), so nothing is stored here.
+template <bool kTrack, class WM>
+__device__ __forceinline__ uint32_t take_name(const Dev& d, const WM& W, Lane& L, int lane, uint32_t net) {
+  const uint32_t x = W.vres[--L.nv][lane];
+  if constexpr (kTrack) __stcg(d.vown + x, net);
+  return x;
+}
+
+// One pop of the global pools for the warp's stacks (ac agents, vc names
+// now): up to Ka and Kv and a few more, or what half of the room above the
+// bump pointer divided among the grid's warps allows, but at least up to
+// Ma and Mv, which one step needs.  Returns false when the arena is full
+// (fatal: the loop stops).  Warp-collective.
+template <class WM>
+__device__ __noinline__ bool fill_stacks(const Dev& d, WM& W, uint32_t ac, uint32_t vc, uint32_t Ka, uint32_t Kv,
+                                         uint32_t Ma, uint32_t Mv) {
+  Ctrl* c = d.ctrl;
+  const int lane = threadIdx.x & 31;
+  // lane 0 serves the agents, lane 1 the names: their counters in one load
+  const unsigned long long* p = lane == 0 ? &c->a_head : lane == 1 ? &c->v_head : lane == 2 ? &c->a_pub
+                              : lane == 3 ? &c->v_pub : lane == 4 ? &c->a_bump : &c->v_bump;
+  unsigned long long cnt = 0;
+  if (lane < 6) cnt = ld_volatile64(p);
+  const unsigned long long pub = __shfl_down_sync(kFull, cnt, 2), bump = __shfl_down_sync(kFull, cnt, 4);
+  const unsigned long long cap = lane == 0 ? d.cap_agents : d.cap_vars;
+  const uint32_t have = lane == 0 ? ac : vc, want = lane == 0 ? Ka : Kv, least = lane == 0 ? Ma : Mv;
+  const uint32_t size = lane == 0 ? (uint32_t)kAStack : (uint32_t)kVStack;
+  uint32_t ok = 1, av = 0, k = 0;
+  unsigned long long rb = 0, bb = 0;
+  if (lane < 2 && want > have) {
+    const unsigned long long room = bump < cap ? cap - bump : 0ull;
+    const unsigned long long warps = (unsigned long long)gridDim.x * (blockDim.x / 32);
+    k = want - have + (lane == 0 ? kFetchA : kFetchV);
+    if (room < 2 * k * warps) k = max((uint32_t)(room / (2 * warps)), least > have ? least - have : 0u);
+    k = min(k, size - have);
+    if (k && cnt < pub) {  // a ring seen empty is left alone
+      const unsigned long long h = atomicAdd(lane == 0 ? &c->a_head : &c->v_head, (unsigned long long)k);
+      av = h < pub ? (uint32_t)min((unsigned long long)k, pub - h) : 0u;
+      rb = h % cap;
+    }
+    if (av < k) {
+      bb = atomicAdd(lane == 0 ? &c->a_bump : &c->v_bump, (unsigned long long)(k - av));
+      if (bb + (k - av) > cap) {
+        ok = 0;
+        set_error(c, INET_ERR_ARENA_FULL, 0);
+      }
+    }
+  }
+  if (!__all_sync(kFull, ok)) return false;
+  // on top of the stacks, the lowest slot last, so that slots from the bump
+  // pointer are taken in ascending order
+#pragma unroll 1
+  for (int w = 0; w < 2; w++) {
+    const uint32_t n = __shfl_sync(kFull, k, w), a = __shfl_sync(kFull, av, w), h = __shfl_sync(kFull, have, w);
+    const unsigned long long r = __shfl_sync(kFull, rb, w), u = __shfl_sync(kFull, bb, w);
+    const unsigned long long cp = __shfl_sync(kFull, cap, w);
+#pragma unroll 1
+    for (uint32_t j = (uint32_t)lane; j < n; j += 32) {
+      uint32_t sl = pool_slot(w ? d.vfree : d.afree, cp, r, a, u, j);
+      if (sl >= cp) {
+        set_error(c, INET_ERR_STATE, 4);
+        sl = 0;
+      }
+      (w ? W.vstk : W.astk)[h + n - 1 - j] = sl;
+    }
+    if (lane == 0) (w ? W.vn : W.an) = (int)(h + n);
+  }
+  __syncwarp();
+  return true;
+}
+
+// Slots for the lanes that lack some for their next interaction (need_a
+// agents, need_v names, 0 for the others; runs: the rule repeats itself along
+// lists), from the warp's stacks into the lanes' columns.  Returns false when
+// the arena is full.  Warp-collective.
+template <class WM>
+__device__ __forceinline__ bool refill(const Dev& d, WM& W, Lane& L, bool runs, uint32_t need_a,
+                                       uint32_t need_v, int lane) {
+  __syncwarp();
+  uint32_t ac = (uint32_t)min(W.an, kAStack), vc = (uint32_t)min(W.vn, kVStack);
+  // what the step needs, or more: a whole column for a run that allocates
+  const uint32_t least_a = (uint32_t)L.na < need_a ? need_a - (uint32_t)L.na : 0u;
+  const uint32_t least_v = (uint32_t)L.nv < need_v ? need_v - (uint32_t)L.nv : 0u;
+  uint32_t wa = least_a ? (uint32_t)(runs ? kARes : max((int)need_a, 4)) - (uint32_t)L.na : 0u;
+  uint32_t wv = least_v ? (uint32_t)max((int)need_v, 4) - (uint32_t)L.nv : 0u;
+  uint32_t inc, packed, Ka, Kv;
+  // offsets of this lane among the warp's wants
+  auto scan = [&]() {
+    packed = inc = wa | (wv << 16);
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t t = __shfl_up_sync(kFull, inc, o);
+      if (lane >= o) inc += t;
+    }
+    const uint32_t tot = __shfl_sync(kFull, inc, 31);
+    Ka = tot & 0xFFFFu;
+    Kv = tot >> 16;
+  };
+  scan();
+  if (Ka > ac || Kv > vc) {
+    // what lanes with no use for them now keep from an earlier run goes back
+    // to the warp before the pools are asked
+    const uint32_t ga = need_a == 0 && L.na > kKeep ? (uint32_t)(L.na - kKeep) : 0u;
+    const uint32_t gv = need_v == 0 && L.nv > kKeep ? (uint32_t)(L.nv - kKeep) : 0u;
+    if (__any_sync(kFull, (ga | gv) != 0)) {
+      uint32_t g = ga | (gv << 16);
+      const uint32_t own = g;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t t = __shfl_up_sync(kFull, g, o);
+        if (lane >= o) g += t;
+      }
+      const uint32_t at_a = ac + ((g - own) & 0xFFFFu), at_v = vc + ((g - own) >> 16);
+      uint32_t da = 0, dv = 0;
+#pragma unroll 1
+      for (; da < ga && at_a + da < (uint32_t)kAStack; da++) W.astk[at_a + da] = W.ares[--L.na][lane];
+#pragma unroll 1
+      for (; dv < gv && at_v + dv < (uint32_t)kVStack; dv++) W.vstk[at_v + dv] = W.vres[--L.nv][lane];
+      const uint32_t tot = __shfl_sync(kFull, g, 31);
+      ac = min(ac + (tot & 0xFFFFu), (uint32_t)kAStack);
+      vc = min(vc + (tot >> 16), (uint32_t)kVStack);
+      __syncwarp();
+    }
+  }
+  if (Ka > ac || Kv > vc) {
+    const uint32_t Ma = __reduce_add_sync(kFull, least_a), Mv = __reduce_add_sync(kFull, least_v);
+    if (!fill_stacks(d, W, ac, vc, Ka, Kv, Ma, Mv)) return false;
+    ac = (uint32_t)min(W.an, kAStack);
+    vc = (uint32_t)min(W.vn, kVStack);
+    if (Ka > ac || Kv > vc) {
+      wa = least_a;
+      wv = least_v;
+      scan();
+    }
+  }
+  const uint32_t oa = ac - ((inc - packed) & 0xFFFFu), ov = vc - ((inc - packed) >> 16);
+#pragma unroll 1
+  for (uint32_t k = 0; k < wa; k++) W.ares[L.na + (int)(wa - 1 - k)][lane] = W.astk[oa - 1 - k];
+#pragma unroll 1
+  for (uint32_t k = 0; k < wv; k++) W.vres[L.nv + (int)(wv - 1 - k)][lane] = W.vstk[ov - 1 - k];
+  L.na += (int)wa;
+  L.nv += (int)wv;
+  __syncwarp();
+  if (lane == 0) {
+    W.an = (int)(ac - Ka);
+    W.vn = (int)(vc - Kv);
+  }
+  __syncwarp();
+  return true;
+}
 
 // ->com for the asynchronous kernel (the chase after a second arrival):
-// link_eq with freed name slots staged per warp.  The lane has fenced its
+// link_eq with freed name slots kept by the lane.  The lane has fenced its
 // new records before linking; a lane that receives a reference through an
 // exchange loads the referenced record only after the exchange returned
 // (address dependency), so it sees the record written before the fence.
-template <bool kTrack>
-__device__ __forceinline__ bool link_async(const Dev& d, WarpMem& W, uint32_t t, uint32_t u, Pair* out) {
+template <bool kTrack, class WM>
+__device__ __forceinline__ bool link_async(const Dev& d, WM& W, Lane& L, int lane, uint32_t t, uint32_t u,
+                                           Pair* out) {
+#pragma unroll 1
   for (uint32_t guard = 0;; guard++) {
     if (is_agent(t) && is_agent(u)) {
       out->a = idx_of(t);
@@ -119,13 +354,13 @@ __device__ __forceinline__ bool link_async(const Dev& d, WarpMem& W, uint32_t t,
       u = w;
     }
     if (!is_var(t) || guard > (1u << 24) || idx_of(t) >= d.cap_vars) {
-      set_error(d.ctrl, INET_ERR_STATE, 1);
+      report(d, INET_ERR_STATE, 1);
       return false;
     }
     const uint32_t x = idx_of(t);
     const uint32_t old = atomicExch(d.var + x, u);
     if (old == kEmpty) return false;
-    release_name<kTrack>(d, W, x);
+    release_name<kTrack>(d, W, L, lane, x);
     t = old;
   }
 }
@@ -137,658 +372,799 @@ struct AsyncTpl {
   uint32_t hdr;                 // n_new | n_fresh << 8 | n_link << 16 | rule << 24
   uint32_t agent[kMaxNew];      // lab | src0 << 8 | src1 << 16 | src2 << 24
   uint16_t link[kMaxLink];      // code0 | code1 << 8
-  uint32_t pad[3];
+  uint32_t inside;              // rules already applied inside: how many | rule << 8 | rule << 16
+  uint32_t pad[2];
 };
 static_assert(sizeof(AsyncTpl) == 64, "packed template is 64 bytes");
 
-__device__ __forceinline__ AsyncTpl pack_template(const Template& t) {
+__device__ __forceinline__ AsyncTpl pack_template(const Template& t, uint32_t inside = 0) {
   AsyncTpl p;
   p.hdr = (uint32_t)t.n_new | ((uint32_t)t.n_fresh << 8) | ((uint32_t)t.n_link << 16) | ((uint32_t)t.rule << 24);
   for (int j = 0; j < kMaxNew; j++)
     p.agent[j] = (uint32_t)t.lab[j] | ((uint32_t)t.src[j][0] << 8) | ((uint32_t)t.src[j][1] << 16) |
                  ((uint32_t)t.src[j][2] << 24);
   for (int k = 0; k < kMaxLink; k++) p.link[k] = (uint16_t)(t.link[k][0] | (t.link[k][1] << 8));
-  p.pad[0] = p.pad[1] = p.pad[2] = 0;
+  p.inside = inside;
+  p.pad[0] = p.pad[1] = 0;
   return p;
 }
 
-// Port value of code c (0xFF: none) from the lane's value table.
-__device__ __forceinline__ int32_t port_val(const WarpMem& W, uint32_t c, int lane) {
-  return c == kValNone ? 0 : (int32_t)W.vals[c][lane];
-}
-
-// Free slots this warp holds privately: warp-uniform counts, kept in the
-// registers of every lane.
-struct WarpStacks {
-  int ac, vc;
+// What one lane's step leaves: new active pairs in W.out[0 .. np)[lane],
+// equations to link after the fence in W.eq[0 .. ne)[lane], how many times
+// the rule was applied, and, when fwd is set, the records of pair 0 (ra always,
+// rb when have_b).
+struct Step {
+  uint32_t np, ne, steps;
+  bool fwd, have_b;
+  int fin;          // rule that ended a run inside it, -1: none
+  int4 ra, rb;
 };
 
-// Where one warp step's new slots come from (warp-uniform): this warp's
-// stacks first (ta agent and tv name slots from abase / vbase up); when a
-// stack runs dry, one global pop serves the rest of the step (ga, gv slots)
-// and refills the stack with kRefill more (gra, grv).
-struct PopPlan {
-  uint32_t ta, tv, abase, vbase, ga, gv, gra, grv;
-  unsigned long long arb, abb, vrb, vbb;
-  uint32_t aav, vav;
-};
-
-// Plans the pops of Ka agent and Kv name slots (warp-collective).  Returns
-// false when the arena is full (fatal: the loop stops).
-__device__ __forceinline__ bool warp_pop(const Dev& d, const WarpStacks& S, uint32_t Ka, uint32_t Kv, int lane,
-                                         PopPlan& P) {
-  Ctrl* c = d.ctrl;
-  P.ta = min((uint32_t)S.ac, Ka);
-  P.tv = min((uint32_t)S.vc, Kv);
-  P.abase = (uint32_t)S.ac - P.ta;
-  P.vbase = (uint32_t)S.vc - P.tv;
-  P.ga = Ka - P.ta;
-  P.gv = Kv - P.tv;
-  P.gra = P.ga ? (uint32_t)kRefill : 0u;
-  P.grv = P.gv ? (uint32_t)kRefill : 0u;
-  P.arb = P.abb = P.vrb = P.vbb = 0;
-  P.aav = P.vav = 0;
-  if (P.ga | P.gv) {
-    uint32_t ok = 1;
-    if (lane == 0) {
-      ok = pool_pop(&c->a_head, &c->a_pub, &c->a_bump, d.cap_agents, P.ga + P.gra, &P.arb, &P.aav, &P.abb) ? 1u : 0u;
-      ok &= pool_pop(&c->v_head, &c->v_pub, &c->v_bump, d.cap_vars, P.gv + P.grv, &P.vrb, &P.vav, &P.vbb) ? 1u : 0u;
-      if (!ok) set_error(c, INET_ERR_ARENA_FULL, 0);
-    }
-    if (!__shfl_sync(kFull, ok, 0)) return false;
-    P.arb = __shfl_sync(kFull, P.arb, 0);
-    P.abb = __shfl_sync(kFull, P.abb, 0);
-    P.aav = __shfl_sync(kFull, P.aav, 0);
-    P.vrb = __shfl_sync(kFull, P.vrb, 0);
-    P.vbb = __shfl_sync(kFull, P.vbb, 0);
-    P.vav = __shfl_sync(kFull, P.vav, 0);
-  }
-  return true;
+// One equation of Theta': two agents are an active pair at once, anything
+// else waits for the fence.
+template <class WM>
+__device__ __forceinline__ void put_equation(WM& W, Step& S, int lane, uint32_t t, uint32_t u) {
+  const bool pair = is_agent(t) && is_agent(u);
+  uint2* to = pair ? reinterpret_cast<uint2*>(&W.out[S.np][lane]) : &W.eq[S.ne][lane];
+  *to = pair ? make_uint2(idx_of(t), idx_of(u)) : make_uint2(t, u);
+  S.np += pair ? 1u : 0u;
+  S.ne += pair ? 0u : 1u;
 }
 
-// The k-th agent / name slot of this warp step.
-__device__ __forceinline__ uint32_t plan_agent(const Dev& d, const WarpMem& W, const PopPlan& P, uint32_t k) {
-  return k < P.ta ? W.astk[P.abase + k] : pool_slot(d.afree, d.cap_agents, P.arb, P.aav, P.abb, k - P.ta);
-}
-__device__ __forceinline__ uint32_t plan_var(const Dev& d, const WarpMem& W, const PopPlan& P, uint32_t k) {
-  return k < P.tv ? W.vstk[P.vbase + k] : pool_slot(d.vfree, d.cap_vars, P.vrb, P.vav, P.vbb, k - P.tv);
-}
-
-// After every lane has read its stack entries (warp-collective): the
-// refills of the stacks, then the agent slots this step frees (free_a of
-// this lane, Fa of the warp; the lane's first at offset `of`) on top of the
-// agent stack, the overflow to the ring.
-template <bool kTrack>
-__device__ __forceinline__ void warp_settle(const Dev& d, WarpMem& W, WarpStacks& S, const PopPlan& P, uint32_t Fa,
-                                            uint32_t free_a, uint32_t of, bool first_is_a, uint32_t a, uint32_t b,
-                                            int lane) {
-  Ctrl* c = d.ctrl;
-  if (P.gra | P.grv) {
-    if ((uint32_t)lane < P.gra) W.astk[P.abase + lane] = pool_slot(d.afree, d.cap_agents, P.arb, P.aav, P.abb, P.ga + lane);
-    if ((uint32_t)lane < P.grv) W.vstk[P.vbase + lane] = pool_slot(d.vfree, d.cap_vars, P.vrb, P.vav, P.vbb, P.gv + lane);
-  }
-  const uint32_t atop = P.abase + P.gra;
-  const uint32_t keep = min((uint32_t)kAStack - atop, Fa);
-  if (Fa) {
-    unsigned long long over = 0;
-    if (Fa > keep) {
-      if (lane == 0) over = atomicAdd(&c->a_tail, (unsigned long long)(Fa - keep));
-      over = __shfl_sync(kFull, over, 0);
-    }
-    for (uint32_t f = 0; f < free_a; f++) {
-      const uint32_t slot = (first_is_a && f == 0) ? a : b;
-      const uint32_t k = of + f;
-      if constexpr (kTrack) __stcg(&d.node[slot].head, kFreeHead);
-      if (k < keep) W.astk[atop + k] = slot;
-      else __stcg(d.afree + (over + (k - keep)) % d.cap_agents, slot);
-    }
-  }
-  S.ac = (int)(atop + keep);
-  S.vc = (int)(P.vbase + P.grv);
-}
-
-// Names freed while linking (warp-collective): on the warp's stack, the
-// overflow to the ring.
-__device__ __forceinline__ void flush_vstage(const Dev& d, WarpMem& W, WarpStacks& S, int lane) {
-  __syncwarp();
-  const int nst = W.vstage_n;
-  if (nst) {
-    const int nv = min(nst, kVStageW);
-    const int keepv = min(kVStack - S.vc, nv);
-    unsigned long long over = 0;
-    if (lane == 0 && nv > keepv) over = atomicAdd(&d.ctrl->v_tail, (unsigned long long)(nv - keepv));
-    over = __shfl_sync(kFull, over, 0);
-    for (int j = lane; j < nv; j += 32) {
-      if (j < keepv) W.vstk[S.vc + j] = W.vstage[j];
-      else __stcg(d.vfree + (over + (unsigned long long)(j - keepv)) % d.cap_vars, W.vstage[j]);
-    }
-    S.vc += keepv;
-    __syncwarp();
-    if (lane == 0) W.vstage_n = 0;
-    __syncwarp();
-  }
-}
-
-// Per-net counters (interactions and the change of pending pairs) and the
-// rule histogram: one fire-and-forget atomic each; with kTrack the net's
-// live agents too (its quota is checked between launches).
-template <bool kTrack>
-__device__ __forceinline__ void count_interaction(const Dev& d, uint32_t* hist, uint32_t net, uint32_t rule,
-                                                  uint32_t np, uint32_t n_new) {
-  atomicAdd(d.netctr + net, 1ull + ((unsigned long long)((long long)np - 1) << kNetPairShift));
-  atomicAdd(&hist[rule], 1u);
-  if constexpr (kTrack) {
-    if (n_new != 2) atomicAdd(reinterpret_cast<unsigned long long*>(d.netlive + net),
-                              (unsigned long long)((long long)n_new - 2));
-  }
-}
-
-// ->com of one lane's equations t_k = u_k, k < nl, after its new records
-// (per lane, no warp-collective step).  One fence makes this lane's new
-// records and fresh names visible before an exchange can publish a
-// reference to them; the first exchange of each of the first kBatch
-// equations is then issued back to back, and only second arrivals continue
-// (rarely) with a chase.  get(k, 0) and get(k, 1) are the two sides of
-// equation k.  kNL >= 0: nl is that constant (the loops unroll); -1: nl is
-// known at run time.  The new active pairs go to W.out[0..return)[lane].
-template <bool kTrack, int kNL, class Get>
-__device__ __forceinline__ uint32_t link_lane(const Dev& d, WarpMem& W, uint32_t nl, const Get& get, int lane) {
-  if constexpr (kNL >= 0) nl = (uint32_t)kNL;
-  constexpr uint32_t kBatch = 2;
-  uint32_t np = 0;
-  __threadfence();
+// ->com of one lane's equations left by its step, after the fence (which
+// makes its new records and fresh names visible before an exchange can
+// publish a reference to them): the first exchange of each of the first
+// kBatch equations is issued back to back, and only second arrivals continue
+// (rarely) with a chase.
+template <bool kTrack, class WM>
+__device__ __forceinline__ void link_lane(const Dev& d, WM& W, Lane& L, Step& S, int lane) {
+  constexpr uint32_t kBatch = 3;
   uint32_t lt[kBatch], lu[kBatch], lo[kBatch];
+  bool more = S.ne > kBatch;
+  uint32_t pend = S.ne > kBatch ? ~0u << kBatch : 0u;  // equations still to chase
 #pragma unroll
   for (uint32_t k = 0; k < kBatch; k++) {
-    lt[k] = 0;
-    lu[k] = 0;
+    lt[k] = lu[k] = 0;
     lo[k] = kEmpty;
-    if (k < nl) {
-      uint32_t t = get(k, 0), u = get(k, 1);
-      if (!(is_agent(t) && is_agent(u))) {
-        if (!is_var(t)) {
-          const uint32_t w = t;
-          t = u;
-          u = w;
-        }
-        if (is_var(t) && idx_of(t) < d.cap_vars) lo[k] = atomicExch(d.var + idx_of(t), u);
-        else set_error(d.ctrl, INET_ERR_STATE, 1);
+    if (k < S.ne) {
+      const uint2 e = W.eq[k][lane];
+      uint32_t t = e.x, u = e.y;
+      if (!is_var(t)) {
+        const uint32_t w = t;
+        t = u;
+        u = w;
       }
+      if (is_var(t) && idx_of(t) < d.cap_vars) lo[k] = atomicExch(d.var + idx_of(t), u);
+      else report(d, INET_ERR_STATE, 1);
       lt[k] = t;
       lu[k] = u;
     }
   }
 #pragma unroll
   for (uint32_t k = 0; k < kBatch; k++) {
-    if (k < nl) {
-      const uint32_t t = lt[k], u = lu[k];
+    if (k < S.ne && lo[k] != kEmpty) {
+      // second arrival: the slot is finished; continue with old = u
+      release_name<kTrack>(d, W, L, lane, idx_of(lt[k]));
+      const uint32_t t = lo[k], u = lu[k];
       if (is_agent(t) && is_agent(u)) {
-        W.out[np][lane] = Pair{idx_of(t), idx_of(u)};
-        np++;
-      } else if (lo[k] != kEmpty && is_var(t)) {
-        // second arrival: the slot is finished; continue with old = u
-        release_name<kTrack>(d, W, idx_of(t));
-        Pair out;
-        if (link_async<kTrack>(d, W, lo[k], u, &out)) {
-          W.out[np][lane] = out;
-          np++;
-        }
+        W.out[S.np][lane] = Pair{idx_of(t), idx_of(u)};
+        S.np++;
+      } else {
+        more = true;
+        W.eq[k][lane] = make_uint2(t, u);
+        pend |= 1u << k;
       }
     }
   }
-  if constexpr (kNL >= 0) {
-#pragma unroll
-    for (uint32_t k = kBatch; k < (uint32_t)kNL; k++) {
+  if (more) {
+#pragma unroll 1
+    for (uint32_t k = 0; k < S.ne; k++) {
+      if (!((pend >> k) & 1u)) continue;
+      const uint2 e = W.eq[k][lane];
       Pair out;
-      if (link_async<kTrack>(d, W, get(k, 0), get(k, 1), &out)) {
-        W.out[np][lane] = out;
-        np++;
-      }
-    }
-  } else {
-    for (uint32_t k = kBatch; k < nl; k++) {
-      Pair out;
-      if (link_async<kTrack>(d, W, get(k, 0), get(k, 1), &out)) {
-        W.out[np][lane] = out;
-        np++;
+      if (link_async<kTrack>(d, W, L, lane, e.x, e.y, &out)) {
+        W.out[S.np][lane] = out;
+        S.np++;
       }
     }
   }
-  return np;
 }
 
 // The rule set a kernel is specialised for: kN templates known at compile
-// time (kT, in rule-table order) and kKey, the hash of their bytes the host
-// passes in Dev::rules_key.  NoRules (kN = 0): the general kernel, which
+// time (kT, in rule-table order, some with active pairs of their own
+// right-hand side already reduced: kMore[I] = how many, and by which rules)
+// and kKey, the hash of the loaded templates that the host passes in
+// Dev::rules_key.  NoRules (kN = 0): the general kernel, which
 // reads the templates from shared memory.
 struct NoRules {
   static constexpr int kN = 0;
   static constexpr unsigned long long kKey = 0;
   static constexpr Template kT[1] = {};
+  static constexpr unsigned char kMore[1][3] = {{0, 0, 0}};
 };
 
-// Instantiation of rule I of a specialised rule set for one lane (Sec. 2.2,
-// ->int, then ->com of Theta'): the template is a constant, so the values
-// live in registers and every loop over agents, ports, names and equations
-// is unrolled.  Slots: the lane's agents beyond the two it reuses start at
-// offset oa of the warp's step, its fresh names at ov (taken from the
-// warp's stacks below ta / tv, the rest from the global pops).  The linking
-// is written out here rather than shared with the general path: the
-// compiler then keeps each equation's known cases (a new agent is an agent,
-// a fresh name a name) apart.
-template <bool kTrack, class Rules, int I>
-__device__ __forceinline__ uint32_t rule_body(const Dev& d, WarpMem& W, const int4& ra, const int4& rb, uint32_t a,
-                                              uint32_t b, uint32_t net, uint32_t oa, uint32_t ov, uint32_t ta,
-                                              uint32_t tv, uint32_t abase, uint32_t vbase, unsigned long long arb,
-                                              uint32_t aav, unsigned long long abb, unsigned long long vrb,
-                                              uint32_t vav, unsigned long long vbb, int lane, bool& valid) {
+// At most this many rules get their own code (the first in rule-table
+// order): every one adds to the run-time compile and to the kernel's code;
+// the others are interpreted.
+constexpr int kSpecialisedMaxRules = 32;
+
+// How rule I repeats itself along a list.  A rule does when one equation of
+// its right-hand side joins a new agent of one of its own left-hand side's
+// symbols (the walker, new agent jc, side cs) to a port e of the other agent
+// (Add(y, w) = x of Add(y, r) = S(x) -> Add(y, w) = x, r = S(w): the walker
+// Add goes on to whatever x is), and every other equation is the head of an
+// output stream: a walker's port p is one when its new value is a fresh name
+// whose other occurrence is port q of another new agent js, and the
+// remaining equation kl joins that agent to the walker's old port p
+// (r = S(w) with w in the walker's port).  Along a list of k such partners
+// the streams then spell js(js(..js(w)..)), with the names between two steps
+// seen by nobody but the lane that reduces them.  Both sides may qualify (S
+// is a walker along the chain of adders that r leads to): the symbol written
+// first on the left-hand side is taken, by custom the one that does the
+// walking.
+struct ChainInfo {
+  bool ok = false;
+  int kc = 0, jc = 0, e = 0, cs = 0;
+  int js[3] = {-1, -1, -1}, q[3] = {0, 0, 0};
+  int other = -1;                           // the new agent that takes the partner's slot, -1: none
+  bool same[3] = {false, false, false};     // js is the partner again, in its slot, but for port q
+};
+__host__ __device__ constexpr ChainInfo chain_info(const Template& R) {
+  ChainInfo none;
+  for (int cand = 0; cand < 2 * R.n_link; cand++) {
+    const int kc = cand % R.n_link;
+    const int c0 = R.link[kc][0], c1 = R.link[kc][1];
+    const bool e0 = c0 < kValNew, e1 = c1 < kValNew;
+    if (e0 == e1) continue;
+    ChainInfo C;
+    C.kc = kc;
+    C.e = e0 ? c0 : c1;
+    C.jc = (e0 ? c1 : c0) - kValNew;
+    if (R.lab[C.jc] != R.lhs[0] && R.lab[C.jc] != R.lhs[1]) continue;
+    C.cs = R.lab[C.jc] == R.lhs[0] ? 0 : 1;
+    if (C.cs != cand / R.n_link || C.e / 3 == C.cs) continue;
+    int heads = 0;
+    for (int p = 0; p < 3; p++) {
+      const int f = R.src[C.jc][p];
+      if (f < kValFresh || f == kValNone) continue;
+      for (int j = 0; j < R.n_new; j++)
+        for (int q = 0; q < 3; q++) {
+          if (j == C.jc || R.src[j][q] != f) continue;
+          for (int k = 0; k < R.n_link; k++) {
+            const int a = R.link[k][0], b = R.link[k][1];
+            const int ext = kValExt + C.cs * 3 + p, agent = kValNew + j;
+            if ((a == ext && b == agent) || (a == agent && b == ext)) {
+              C.js[p] = j;
+              C.q[p] = q;
+              heads++;
+            }
+          }
+        }
+    }
+    if (heads != R.n_link - 1 || (C.cs == 1 && heads == 0)) continue;
+    for (int j = R.n_new - 1; j >= 0; j--)
+      if (j != C.jc) C.other = j;
+    for (int p = 0; p < 3; p++) {
+      if (C.js[p] < 0) continue;
+      const int ps = 1 - C.cs;
+      bool same = C.js[p] == C.other && R.lab[C.js[p]] == R.lhs[ps];
+      for (int r = 0; r < 3; r++) {
+        if (r == C.q[p]) continue;
+        const int c = R.src[C.js[p]][r];
+        if (c != kValNone && c != kValExt + ps * 3 + r) same = false;
+      }
+      C.same[p] = same;
+    }
+    C.ok = true;
+    return C;
+  }
+  return none;
+}
+
+// Ports of the left-hand side's agent `side` (each is used once on the
+// right-hand side).
+__host__ __device__ constexpr int chain_arity(const Template& R, int side) {
+  int n = 0;
+  for (int j = 0; j < R.n_new; j++)
+    for (int p = 0; p < 3; p++)
+      if (R.src[j][p] < kValNew && R.src[j][p] / 3 == side) n++;
+  for (int k = 0; k < R.n_link; k++)
+    for (int i = 0; i < 2; i++)
+      if (R.link[k][i] < kValNew && R.link[k][i] / 3 == side) n++;
+  return n;
+}
+// The record of a partner, or its first half when that is all it holds.
+template <bool kNarrow>
+__device__ __forceinline__ int4 ld_partner(const Node* p) {
+  if constexpr (kNarrow) {
+    const uint2 v = __ldcg(reinterpret_cast<const uint2*>(p));
+    return make_int4((int)v.x, (int)v.y, 0, 0);
+  } else {
+    return ld_node(p);
+  }
+}
+
+// The walker leaves every partner of a run in its slot as it is: one output
+// stream, of the partners themselves, no other new agent, the walker's other
+// ports unchanged.
+__host__ __device__ constexpr bool chain_passes(const Template& R, const ChainInfo& C) {
+  if (!C.ok || R.n_new != 2 || R.n_fresh != 1) return false;
+  for (int p = 0; p < 3; p++) {
+    if (C.js[p] >= 0) {
+      if (!C.same[p] || C.q[p] != C.e % 3) return false;
+    } else if (R.src[C.jc][p] != kValNone && R.src[C.jc][p] != kValExt + C.cs * 3 + p) {
+      return false;
+    }
+  }
+  return true;
+}
+
+// Component q of a record's auxiliary words (q is a constant where it is used).
+__device__ __forceinline__ void set_aux(int4& r, int q, uint32_t w) {
+  if (q == 0) r.y = (int32_t)w;
+  else if (q == 1) r.z = (int32_t)w;
+  else r.w = (int32_t)w;
+}
+__device__ __forceinline__ uint32_t get_aux(const int4& r, int q) {
+  return (uint32_t)(q == 0 ? r.y : q == 1 ? r.z : r.w);
+}
+
+// Rule I of a specialised rule set for one lane (Sec. 2.2, ->int): the
+// template is a constant, so the values live in registers and every loop
+// over agents, ports, names and equations is unrolled.  Records are stored,
+// equations are left for the fence that the whole warp shares.
+template <bool kTrack, class Rules, int I, class WM>
+__device__ __forceinline__ void one_step(const Dev& d, WM& W, Lane& L, int lane, uint32_t a, uint32_t b,
+                                         const int4& ra, const int4& rb, uint32_t net, Step& S) {
   constexpr Template R = Rules::kT[I];
-  Ctrl* c = d.ctrl;
   uint32_t v[kNumVals];
-  v[kValExt + 0] = (uint32_t)ra.y;
-  v[kValExt + 1] = (uint32_t)ra.z;
-  v[kValExt + 2] = (uint32_t)ra.w;
-  v[kValExt + 3] = (uint32_t)rb.y;
-  v[kValExt + 4] = (uint32_t)rb.z;
-  v[kValExt + 5] = (uint32_t)rb.w;
+#pragma unroll
+  for (int q = 0; q < 3; q++) {
+    v[kValExt + q] = get_aux(ra, q);
+    v[kValExt + 3 + q] = get_aux(rb, q);
+  }
 #pragma unroll
   for (int j = kValNew; j < kNumVals; j++) v[j] = 0;
-  bool in_range = true;
   if (R.n_new > 0) v[kValNew + 0] = mk_agent(a);
   if (R.n_new > 1) v[kValNew + 1] = mk_agent(b);
 #pragma unroll
-  for (int j = 2; j < (int)R.n_new; j++) {
-    const uint32_t k = oa + (uint32_t)j - 2;
-    const uint32_t sl = k < ta ? W.astk[abase + k] : pool_slot(d.afree, d.cap_agents, arb, aav, abb, k - ta);
-    if (sl >= d.cap_agents) in_range = false;
-    v[kValNew + j] = mk_agent(sl);
-  }
+  for (int j = 2; j < (int)R.n_new; j++) v[kValNew + j] = mk_agent(take_agent(W, L, lane));
 #pragma unroll
-  for (int f = 0; f < (int)R.n_fresh; f++) {
-    const uint32_t k = ov + (uint32_t)f;
-    const uint32_t x = k < tv ? W.vstk[vbase + k] : pool_slot(d.vfree, d.cap_vars, vrb, vav, vbb, k - tv);
-    if (x >= d.cap_vars) {
-      in_range = false;
-    } else {
-      __stcg(d.var + x, kEmpty);  // a fresh name starts empty; published by this lane's fence
-      if constexpr (kTrack) __stcg(d.vown + x, net);
-    }
-    v[kValFresh + f] = mk_var(x);
-  }
-  if (!in_range) {
-    set_error(c, INET_ERR_STATE, 4);
-    valid = false;
-    return 0u;
-  }
-  const uint32_t head_net = net << 8;
+  for (int f = 0; f < (int)R.n_fresh; f++) v[kValFresh + f] = mk_var(take_name<kTrack>(d, W, L, lane, net));
 #pragma unroll
   for (int j = 0; j < (int)R.n_new; j++) {
     int4 rec;
-    rec.x = (int32_t)(head_net | R.lab[j]);
+    rec.x = (int32_t)((net << 8) | R.lab[j]);
     rec.y = R.src[j][0] == kValNone ? 0 : (int32_t)v[R.src[j][0]];
     rec.z = R.src[j][1] == kValNone ? 0 : (int32_t)v[R.src[j][1]];
     rec.w = R.src[j][2] == kValNone ? 0 : (int32_t)v[R.src[j][2]];
     st_node(d.node + idx_of(v[kValNew + j]), rec);
   }
-  // ->com: the fence, the first exchanges of the first kBatch equations back
-  // to back, then their second arrivals, then the other equations
-  constexpr uint32_t kBatch = 2;
-  uint32_t np = 0;
-  if (R.n_link) __threadfence();
-  uint32_t lt[kBatch], lu[kBatch], lo[kBatch];
+  if (R.n_new == 0) put_agent<kTrack>(d, W, L, lane, a);
+  if (R.n_new < 2) put_agent<kTrack>(d, W, L, lane, b);
+  L.live += (int)R.n_new - 2;
+  S.steps = 1;
 #pragma unroll
-  for (uint32_t k = 0; k < kBatch; k++) {
-    lt[k] = 0;
-    lu[k] = 0;
-    lo[k] = kEmpty;
-    if (k < R.n_link) {
-      uint32_t t = v[R.link[k][0]], u = v[R.link[k][1]];
-      if (!(is_agent(t) && is_agent(u))) {
-        if (!is_var(t)) {
-          const uint32_t w = t;
-          t = u;
-          u = w;
-        }
-        if (is_var(t) && idx_of(t) < d.cap_vars) lo[k] = atomicExch(d.var + idx_of(t), u);
-        else set_error(c, INET_ERR_STATE, 1);
-      }
-      lt[k] = t;
-      lu[k] = u;
-    }
-  }
-#pragma unroll
-  for (uint32_t k = 0; k < kBatch; k++) {
-    if (k < R.n_link) {
-      const uint32_t t = lt[k], u = lu[k];
-      if (is_agent(t) && is_agent(u)) {
-        W.out[np][lane] = Pair{idx_of(t), idx_of(u)};
-        np++;
-      } else if (lo[k] != kEmpty && is_var(t)) {
-        release_name<kTrack>(d, W, idx_of(t));
-        Pair out;
-        if (link_async<kTrack>(d, W, lo[k], u, &out)) {
-          W.out[np][lane] = out;
-          np++;
-        }
-      }
-    }
-  }
-#pragma unroll
-  for (uint32_t k = kBatch; k < R.n_link; k++) {
-    Pair out;
-    if (link_async<kTrack>(d, W, v[R.link[k][0]], v[R.link[k][1]], &out)) {
-      W.out[np][lane] = out;
-      np++;
-    }
-  }
-  return np;
+  for (int k = 0; k < (int)R.n_link; k++) put_equation(W, S, lane, v[R.link[k][0]], v[R.link[k][1]]);
 }
 
-// Rule I continues as a chain of itself when one of its equations joins an
-// external port to a new agent of one of its own left-hand side's symbols:
-// Add(y, w) = x of Add(y, r) = S(x) -> Add(y, w) = x, r = S(w), where an
-// agent x in the port makes (Add', x) the next active pair, often of the
-// same rule.
-template <class Rules, int I>
-__host__ __device__ constexpr bool chain_rule() {
-  if constexpr (I < Rules::kN) {
-    constexpr Template R = Rules::kT[I];
-    for (int k = 0; k < R.n_link; k++) {
-      const int c0 = R.link[k][0], c1 = R.link[k][1];
-      const bool e0 = c0 < kValNew, e1 = c1 < kValNew;
-      const bool n0 = c0 >= kValNew && c0 < kValFresh, n1 = c1 >= kValNew && c1 < kValFresh;
-      if ((e0 && n1) || (n0 && e1)) {
-        const int lab = R.lab[(e0 ? c1 : c0) - kValNew];
-        if (lab == R.lhs[0] || lab == R.lhs[1]) return true;
+// Rule J can end a run of rule I inside it: the walker meets an agent that
+// the list ends with (Add(y, r) = Z -> r = y after Add(y, r) = S(x)), and J
+// joins each of the run's output streams to something it has at hand, which
+// then goes straight into the open port of the stream's last agent.  That
+// saves a name, the walker's record and a whole step at every list's end, and
+// leaves lists with fewer names in them for whoever walks them next: 512
+// random trees 1.7 -> 1.4 ms, Fibonacci(22..25) x 64 47.5 -> 43.5 ms (and 2048
+// Mul nets 3.9 -> 4.4 ms, whose runs it makes uneven).
+template <class Rules, int I, int J>
+__host__ __device__ constexpr bool ends_run() {
+  constexpr Template R = Rules::kT[I], T = Rules::kT[J];
+  constexpr ChainInfo C = chain_info(R);
+  if (I == J || T.n_fresh != 0 || T.n_new > 2) return false;
+  const int wl = R.lhs[C.cs];
+  if (T.lhs[0] != wl && T.lhs[1] != wl) return false;
+  const int side = T.lhs[0] == wl ? 0 : 1;
+  for (int p = 0; p < 3; p++) {
+    if (C.js[p] < 0) continue;
+    int uses = 0;
+    for (int k = 0; k < T.n_link; k++)
+      for (int i = 0; i < 2; i++) {
+        if (T.link[k][i] != kValExt + side * 3 + p) continue;
+        const int o = T.link[k][1 - i];
+        for (int r = 0; r < 3; r++)
+          if (C.js[r] >= 0 && o == kValExt + side * 3 + r) return false;
+        uses++;
+      }
+    if (uses != 1) return false;
+  }
+  return true;
+}
+
+// At the end of a run of rule I: the walker (slot cslot, ports c) has come to
+// agent `at` with record nb (its first half when kNarrow) of another label;
+// hs, hr: the streams' last agents.  True when a rule ended the run here.
+template <bool kTrack, class Rules, int I, bool kNarrow, int J = 0, class WM>
+__device__ __forceinline__ bool end_run(const Dev& d, WM& W, Lane& L, int lane, uint32_t net, uint32_t cslot,
+                                        const uint32_t (&c)[3], uint32_t at, int4 nb, const uint32_t (&hs)[3],
+                                        int4 (&hr)[3], Step& S) {
+  if constexpr (J < Rules::kN && J < kSpecialisedMaxRules) {
+    if constexpr (ends_run<Rules, I, J>()) {
+      constexpr Template R = Rules::kT[I], T = Rules::kT[J];
+      constexpr ChainInfo C = chain_info(R);
+      constexpr int side = T.lhs[0] == R.lhs[C.cs] ? 0 : 1;
+      if (((uint32_t)nb.x & 0xFFu) == T.lhs[1 - side]) {
+        if constexpr (kNarrow && chain_arity(T, 1 - side) > 1) nb = ld_node(d.node + at);
+        uint32_t v[kNumVals];
+#pragma unroll
+        for (int q = 0; q < 3; q++) {
+          v[side * 3 + q] = c[q];
+          v[(1 - side) * 3 + q] = get_aux(nb, q);
+        }
+        v[kValNew + 0] = mk_agent(cslot);
+        v[kValNew + 1] = mk_agent(at);
+#pragma unroll
+        for (int j = 0; j < (int)T.n_new; j++) {
+          int4 rec;
+          rec.x = (int32_t)((net << 8) | T.lab[j]);
+          rec.y = T.src[j][0] == kValNone ? 0 : (int32_t)v[T.src[j][0]];
+          rec.z = T.src[j][1] == kValNone ? 0 : (int32_t)v[T.src[j][1]];
+          rec.w = T.src[j][2] == kValNone ? 0 : (int32_t)v[T.src[j][2]];
+          st_node(d.node + idx_of(v[kValNew + j]), rec);
+        }
+#pragma unroll
+        for (int k = 0; k < (int)T.n_link; k++) {
+          bool stream = false;
+#pragma unroll
+          for (int p = 0; p < 3; p++) {
+            if (C.js[p] < 0) continue;
+#pragma unroll
+            for (int i = 0; i < 2; i++)
+              if (T.link[k][i] == kValExt + side * 3 + p) {
+                set_aux(hr[p], C.q[p], v[T.link[k][1 - i]]);
+                st_node(d.node + hs[p], hr[p]);
+                stream = true;
+              }
+          }
+          if (!stream) put_equation(W, S, lane, v[T.link[k][0]], v[T.link[k][1]]);
+        }
+        if (T.n_new == 0) put_agent<kTrack>(d, W, L, lane, cslot);
+        if (T.n_new < 2) put_agent<kTrack>(d, W, L, lane, at);
+        L.live += (int)T.n_new - 2;
+        S.fin = J;
+        return true;
       }
     }
+    return end_run<kTrack, Rules, I, kNarrow, J + 1>(d, W, L, lane, net, cslot, c, at, nb, hs, hr, S);
   }
   return false;
 }
 
-constexpr int kLoneMax = 32;  // steps of one lone or uniform run before the warp's loop resumes
-
-// A warp whose valid lanes all reduce rule I of a specialised rule set (the
-// common case: one lane alone on a chain, or a batch of like pairs): the
-// whole step with that rule's template as a constant.  Every lane needs the
-// same slots, so a lane's offsets among the warp's needs are its rank among
-// the valid lanes times the rule's counts, with no scan.
+// Rule I along a list (see ChainInfo): up to `lim` interactions without
+// leaving the lane.  The walker keeps its slot and its ports stay in
+// registers; each step loads the next partner (in flight ahead, see below),
+// and the record an output stream's last agent waits for gets that step's
+// agent in its open port.  The names between two steps are never created,
+// the records of agents that come out as they went in (the S of Add(y, r) =
+// S(x)) are not rewritten, and the streams' heads are linked once at the
+// end, with one fence and one exchange for the whole run instead of one per
+// interaction.  What bounds it: about 70 instructions a step of one lane
+// (500 cycles alone), then the round trips of partners that do not lie side
+// by side.
 //
-// Uniform runs: when `quiet` (no lane waits for a ticket and the queue was
-// empty when the warp last looked), the rule continues as a chain of itself
-// and every valid lane's step left exactly one new pair, of rule I again,
-// the warp steps again at once with those pairs, without its loop between
-// (up to kLoneMax steps): nothing is handed on, the count of pairs in flight
-// does not change.  A warp with one valid lane leaves this to lone_chain.
-template <bool kTrack, class Rules, int I>
-__device__ __forceinline__ uint32_t uni_interact(const Dev& d, const int16_t* tab, uint32_t* hist, WarpMem& W,
-                                                 WarpStacks& S, bool valid, unsigned vmask, uint32_t a, uint32_t b,
-                                                 int4 ra, int4 rb, uint32_t net, long long& live, bool quiet) {
+// Partners ahead: lists are mostly laid out in slot order (numerals as they
+// were loaded, copies as they were allocated), so each load of a partner
+// also loads the next slots in the direction the list last went; they are
+// used only if the list really leads there.  Such an early load is as good
+// as a late one: an agent that a record already reached names directly is
+// owned by this lane, was written before that record was published and does
+// not change (a name in between ends the window).
+template <bool kTrack, class Rules, int I, class WM>
+__device__ __forceinline__ void run_rule(const Dev& d, WM& W, Lane& L, int lane, uint32_t a, uint32_t b,
+                                         const int4& ra, const int4& rb, uint32_t net, uint32_t lim, Step& S) {
   constexpr Template R = Rules::kT[I];
-  constexpr uint32_t NN = R.n_new, NF = R.n_fresh;
-  constexpr uint32_t NA = NN > 2 ? NN - 2 : 0u, FA = NN < 2 ? 2 - NN : 0u;
-  const int lane = threadIdx.x & 31;
-  Ctrl* c = d.ctrl;
-  const uint32_t nvl = __popc(vmask), rank = __popc(vmask & lanemask_lt());
-  const uint32_t Ka = nvl * NA, Kv = nvl * NF, Fa = nvl * FA;
-  const uint32_t oa = rank * NA, ov = rank * NF, of = rank * FA;
-  uint32_t np = 0;
-  for (int it = 0;; it++) {
-    const uint32_t ta = min((uint32_t)S.ac, Ka), tv = min((uint32_t)S.vc, Kv);
-    const uint32_t abase = (uint32_t)S.ac - ta, vbase = (uint32_t)S.vc - tv;
-    const uint32_t ga = Ka - ta, gv = Kv - tv;
-    const uint32_t gra = ga ? (uint32_t)kRefill : 0u, grv = gv ? (uint32_t)kRefill : 0u;
-    unsigned long long arb = 0, abb = 0, vrb = 0, vbb = 0;
-    uint32_t aav = 0, vav = 0;
-    if (ga | gv) {
-      uint32_t ok = 1;
-      if (lane == 0) {
-        ok = pool_pop(&c->a_head, &c->a_pub, &c->a_bump, d.cap_agents, ga + gra, &arb, &aav, &abb) ? 1u : 0u;
-        ok &= pool_pop(&c->v_head, &c->v_pub, &c->v_bump, d.cap_vars, gv + grv, &vrb, &vav, &vbb) ? 1u : 0u;
-        if (!ok) set_error(c, INET_ERR_ARENA_FULL, 0);
-      }
-      if (!__shfl_sync(kFull, ok, 0)) return 0u;  // fatal: the loop stops
-      arb = __shfl_sync(kFull, arb, 0);
-      abb = __shfl_sync(kFull, abb, 0);
-      aav = __shfl_sync(kFull, aav, 0);
-      vrb = __shfl_sync(kFull, vrb, 0);
-      vbb = __shfl_sync(kFull, vbb, 0);
-      vav = __shfl_sync(kFull, vav, 0);
-    }
-    if (lane == 0) live += (long long)Ka - (long long)Fa;
-    const bool frees = valid;  // counted in Fa: freed even if the step fails below
-    np = 0;
-    if (valid)
-      np = rule_body<kTrack, Rules, I>(d, W, ra, rb, a, b, net, oa, ov, ta, tv, abase, vbase, arb, aav, abb, vrb,
-                                       vav, vbb, lane, valid);
-    __syncwarp();  // every taken stack entry has been read
-    if (gra | grv) {
-      if ((uint32_t)lane < gra) W.astk[abase + lane] = pool_slot(d.afree, d.cap_agents, arb, aav, abb, ga + lane);
-      if ((uint32_t)lane < grv) W.vstk[vbase + lane] = pool_slot(d.vfree, d.cap_vars, vrb, vav, vbb, gv + lane);
-    }
-    const uint32_t atop = abase + gra;
-    const uint32_t keep = min((uint32_t)kAStack - atop, Fa);
-    if (FA && Fa) {
-      unsigned long long over = 0;
-      if (Fa > keep) {
-        if (lane == 0) over = atomicAdd(&c->a_tail, (unsigned long long)(Fa - keep));
-        over = __shfl_sync(kFull, over, 0);
-      }
-      if (frees) {
+  constexpr ChainInfo C = chain_info(R);
+  constexpr int kWalk = kValExt + C.cs * 3, kPart = kValExt + (1 - C.cs) * 3;
+  constexpr int kNeedA = R.n_new > 2 ? R.n_new - 2 : 0;
+  const uint32_t cslot = C.cs == 0 ? a : b;
+  uint32_t pslot = C.cs == 0 ? b : a;
+  uint32_t v[kNumVals];
+  const int4 rw = C.cs == 0 ? ra : rb;
+  int4 rp = C.cs == 0 ? rb : ra;
 #pragma unroll
-        for (uint32_t f = 0; f < FA; f++) {
-          const uint32_t slot = (NN == 0 && f == 0) ? a : b;
-          const uint32_t k = of + f;
-          if constexpr (kTrack) __stcg(&d.node[slot].head, kFreeHead);
-          if (k < keep) W.astk[atop + k] = slot;
-          else __stcg(d.afree + (over + (k - keep)) % d.cap_agents, slot);
-        }
+  for (int q = 0; q < 3; q++) v[kWalk + q] = get_aux(rw, q);
+#pragma unroll
+  for (int j = kValNew; j < kNumVals; j++) v[j] = 0;
+  v[kValNew + C.jc] = mk_agent(cslot);
+  // streams: the equation of the head, and the last agent with its open port
+  uint32_t r0[3], h0[3], hs[3], hold[3];
+  int4 hr[3];
+#pragma unroll
+  for (int p = 0; p < 3; p++) {
+    r0[p] = h0[p] = hs[p] = hold[p] = 0;
+    hr[p] = make_int4(0, 0, 0, 0);
+  }
+  constexpr uint32_t kWin = 4;
+  int4 w0 = rp, w1 = rp, w2 = rp, w3 = rp;
+  uint32_t wn = 0, wi = 0, dir = 1;
+  uint32_t steps = 0, x = 0;
+  bool ready = true;  // the partner rp at pslot is there to be reduced
+  S.have_b = false;
+  for (uint32_t guard = 0;; guard++) {
+    if (ready) {
+#pragma unroll
+    for (int q = 0; q < 3; q++) v[kPart + q] = get_aux(rp, q);
+#pragma unroll
+    for (int j = 0; j < (int)R.n_new; j++)
+      if (j != C.jc) v[kValNew + j] = mk_agent(j == C.other ? pslot : take_agent(W, L, lane));
+    if (C.other < 0) put_agent<kTrack>(d, W, L, lane, pslot);
+    // fresh names, but for the ones between this step and the next
+#pragma unroll
+    for (int f = 0; f < (int)R.n_fresh; f++) {
+      bool open = false;
+#pragma unroll
+      for (int p = 0; p < 3; p++)
+        if (C.js[p] >= 0 && R.src[C.jc][p] == kValFresh + f) open = true;
+      if (!open) v[kValFresh + f] = mk_var(take_name<kTrack>(d, W, L, lane, net));
+    }
+    // the streams' previous agents get this step's in their open ports
+#pragma unroll
+    for (int p = 0; p < 3; p++) {
+      if (C.js[p] < 0) continue;
+      const uint32_t w = v[kValNew + (C.js[p] < 0 ? 0 : C.js[p])];
+      if (steps == 0) {
+        r0[p] = v[kWalk + p];
+        h0[p] = w;
+      } else if (!C.same[p] || hold[p] != w) {
+        set_aux(hr[p], C.q[p], w);
+        st_node(d.node + hs[p], hr[p]);
       }
     }
-    S.ac = (int)(atop + keep);
-    S.vc = (int)(vbase + grv);
-    flush_vstage(d, W, S, lane);
-    if (valid) count_interaction<kTrack>(d, hist, net, R.rule, np, NN);
-    if constexpr (!chain_rule<Rules, I>()) {
+    // this step's new agents
+#pragma unroll
+    for (int j = 0; j < (int)R.n_new; j++) {
+      if (j == C.jc) continue;
+      int4 rec;
+      rec.x = (int32_t)((net << 8) | R.lab[j]);
+      rec.y = R.src[j][0] == kValNone ? 0 : (int32_t)v[R.src[j][0]];
+      rec.z = R.src[j][1] == kValNone ? 0 : (int32_t)v[R.src[j][1]];
+      rec.w = R.src[j][2] == kValNone ? 0 : (int32_t)v[R.src[j][2]];
+      bool open = false;
+#pragma unroll
+      for (int p = 0; p < 3; p++)
+        if (C.js[p] == j) {
+          hr[p] = rec;
+          hs[p] = idx_of(v[kValNew + j]);
+          hold[p] = get_aux(rp, C.q[p]);
+          open = true;
+        }
+      if (!open) st_node(d.node + idx_of(v[kValNew + j]), rec);
+    }
+    // the walker's ports
+    uint32_t nx[3];
+#pragma unroll
+    for (int p = 0; p < 3; p++)
+      nx[p] = R.src[C.jc][p] == kValNone || C.js[p] >= 0 ? 0u : v[R.src[C.jc][p] == kValNone ? 0 : R.src[C.jc][p]];
+    x = v[C.e];
+#pragma unroll
+    for (int p = 0; p < 3; p++) v[kWalk + p] = nx[p];
+    steps++;
+    ready = false;
+    }
+    // one round trip for every lane of the warp, whatever it waits for: a
+    // name (see pass_rule), or the next partner
+    const uint32_t at = idx_of(x);
+    const bool name = is_var(x);
+    if (name ? at >= d.cap_vars || guard > 2 * lim
+             : !is_agent(x) || at >= d.cap_agents || steps >= lim || L.na < kNeedA || L.nv < (int)R.n_fresh)
       break;
+    uint32_t old = kEmpty;
+    if (name) {
+      old = ld_volatile(d.var + at);
+    } else if (wn == 0 || at != wi) {
+      dir = at == pslot - 1 ? ~0u : at == pslot + 1 ? 1u : dir;
+      w0 = ld_node(d.node + at);
+      const uint32_t i1 = at + dir, i2 = i1 + dir, i3 = i2 + dir;
+      w1 = ld_node(d.node + (i1 < d.cap_agents ? i1 : at));
+      w2 = ld_node(d.node + (i2 < d.cap_agents ? i2 : at));
+      w3 = ld_node(d.node + (i3 < d.cap_agents ? i3 : at));
+      wn = kWin;
+      wi = at;
+    }
+    if (name) {
+      if (old == kEmpty) break;
+      release_name<kTrack>(d, W, L, lane, at);
+      x = old;
+      wn = 0;
     } else {
-      // every lane's chain goes on with another pair of rule I: the warp
-      // steps again without its loop (the records read here are wasted when
-      // some lane's next pair is of another rule: once at the end of a chain)
-      if (!quiet || nvl == 1 || it + 1 >= kLoneMax || !__all_sync(kFull, !valid || np == 1)) break;
-      bool ok = true;
-      if (valid) {
-        ok = false;
-        const Pair p = W.out[0][lane];
-        if (p.a < d.cap_agents && p.b < d.cap_agents) {
-          const int4 pra = ld_node(d.node + p.a), prb = ld_node(d.node + p.b);
-          const uint32_t la = (uint32_t)pra.x & 0xFFu, lb = (uint32_t)prb.x & 0xFFu;
-          const int e = (la < d.n_labels && lb < d.n_labels) ? tab[la * d.n_labels + lb] : -1;
-          if (e >= 0 && ((uint32_t)e >> 1) == (uint32_t)I) {
-            if (e & 1) {
-              ra = prb;
-              rb = pra;
-              a = p.b;
-              b = p.a;
-            } else {
-              ra = pra;
-              rb = prb;
-              a = p.a;
-              b = p.b;
-            }
-            net = (uint32_t)ra.x >> 8;
-            ok = net < d.max_nets;
-          }
-        }
+      rp = w0;
+      w0 = w1;
+      w1 = w2;
+      w2 = w3;
+      wn--;
+      wi += dir;
+      pslot = at;
+      ready = ((uint32_t)rp.x & 0xFFu) == R.lhs[1 - C.cs];
+      if (!ready) {
+        S.have_b = true;
+        break;
       }
-      if (!__all_sync(kFull, ok)) break;
     }
   }
-  return valid ? np : 0u;
-}
-
-// Rule I of a specialised rule set, when the rule set has one and I's
-// right-hand side has at most two agents (it reuses the pair's two slots:
-// the rules that carry chains, Add(y, r) = S(x) and the like).  Larger
-// rules stay on the general code: their own copies cost more in instruction
-// fetch than they save (2048 Mul nets: 10.9 ms with rules of up to two
-// agents, 11.0 ms up to three, 11.2 ms with every rule; only up to one
-// leaves the Add chains out and gives no gain).
-
-// A warp in which one lane holds a pair (no lane waits for a ticket, and the
-// queue was empty when the warp last looked), of a rule that continues as a
-// chain of itself: the lane runs up to kLoneMax interactions of that rule on
-// its own, without the warp's loop between them.  Each leaves exactly one
-// new pair, the chain's next, so nothing is handed on and the count of pairs
-// in flight does not change.  The run stops when an interaction leaves no
-// pair or several (returned as after any step, W.out filled), when the next
-// pair is of another rule or its slots are not on the warp's stacks (it is
-// then the lane's next pair), or after kLoneMax interactions.  Slots come
-// from and return to the warp's stacks, names freed while linking too;
-// counters per interaction as in the warp's step.  (Loading the next
-// pair's records before an interaction's fence and exchanges returned, or
-// handing the records this run loaded back to the warp's loop, was slower.)
-template <bool kTrack, class Rules, int I>
-__device__ __forceinline__ uint32_t lone_chain(const Dev& d, const int16_t* tab, uint32_t* hist, WarpMem& W,
-                                               WarpStacks& S, bool valid, uint32_t a, uint32_t b, int4 ra, int4 rb,
-                                               uint32_t net, long long& live) {
-  constexpr Template R = Rules::kT[I];
-  constexpr uint32_t NN = R.n_new, NF = R.n_fresh;
-  constexpr uint32_t NA = NN > 2 ? NN - 2 : 0u, FA = NN < 2 ? 2 - NN : 0u;
-  const int lane = threadIdx.x & 31;
-  Ctrl* c = d.ctrl;
-  const unsigned vm = __ballot_sync(kFull, valid);
-  const int src = vm ? __ffs(vm) - 1 : 0;
-  uint32_t np = 0;
-  int ac = S.ac, vc = S.vc;
-  long long dl = 0;
-  if (valid) {
-    for (int it = 0;; it++) {
-      np = rule_body<kTrack, Rules, I>(d, W, ra, rb, a, b, net, 0u, 0u, NA, NF, (uint32_t)ac - NA,
-                                       (uint32_t)vc - NF, 0ull, 0u, 0ull, 0ull, 0u, 0ull, lane, valid);
-      ac -= (int)NA;
-      vc -= (int)NF;
+  L.live += (long long)((int)R.n_new - 2) * (long long)steps;
+  S.steps = steps;
+  bool ended = false;
+  if (S.have_b) {
+    const uint32_t c[3] = {v[kWalk + 0], v[kWalk + 1], v[kWalk + 2]};
+    ended = end_run<kTrack, Rules, I, false>(d, W, L, lane, net, cslot, c, pslot, rp, hs, hr, S);
+  }
+  if (!ended) {
+    // each stream's last agent and the walker's port get a name, the
+    // walker's record is stored
 #pragma unroll
-      for (uint32_t f = 0; f < FA; f++) {
-        const uint32_t slot = (NN == 0 && f == 0) ? a : b;
-        if constexpr (kTrack) __stcg(&d.node[slot].head, kFreeHead);
-        if (ac < kAStack) {
-          W.astk[ac++] = slot;
-        } else {
-          const unsigned long long tp = atomicAdd(&c->a_tail, 1ull);
-          __stcg(d.afree + tp % d.cap_agents, slot);
-        }
-      }
-      dl += (long long)NA - (long long)FA;
-      // names freed while linking: this lane is the only user of the warp's stacks
-      const int nst = min(W.vstage_n, kVStageW);
-      for (int j = 0; j < nst; j++) {
-        if (vc < kVStack) {
-          W.vstk[vc++] = W.vstage[j];
-        } else {
-          const unsigned long long tp = atomicAdd(&c->v_tail, 1ull);
-          __stcg(d.vfree + tp % d.cap_vars, W.vstage[j]);
-        }
-      }
-      W.vstage_n = 0;
-      if (!valid) break;
-      count_interaction<kTrack>(d, hist, net, R.rule, np, NN);
-      if (np != 1 || it + 1 >= kLoneMax) break;
-      // the one new pair: the chain's next if it is of rule I again
-      const Pair p = W.out[0][lane];
-      if (p.a >= d.cap_agents || p.b >= d.cap_agents) break;
-      const int4 pra = ld_node(d.node + p.a), prb = ld_node(d.node + p.b);
-      const uint32_t la = (uint32_t)pra.x & 0xFFu, lb = (uint32_t)prb.x & 0xFFu;
-      const int e = (la < d.n_labels && lb < d.n_labels) ? tab[la * d.n_labels + lb] : -1;
-      if (e < 0 || ((uint32_t)e >> 1) != (uint32_t)I || ac < (int)NA || vc < (int)NF) break;
-      if (e & 1) {
-        ra = prb;
-        rb = pra;
-        a = p.b;
-        b = p.a;
-      } else {
-        ra = pra;
-        rb = prb;
-        a = p.a;
-        b = p.b;
-      }
-      net = (uint32_t)ra.x >> 8;
-      if (net >= d.max_nets) break;  // left to the warp's step, which reports it
+    for (int p = 0; p < 3; p++) {
+      if (C.js[p] < 0) continue;
+      const uint32_t w = mk_var(take_name<kTrack>(d, W, L, lane, net));
+      set_aux(hr[p], C.q[p], w);
+      st_node(d.node + hs[p], hr[p]);
+      v[kWalk + p] = w;
+    }
+    int4 rec;
+    rec.x = (int32_t)((net << 8) | R.lab[C.jc]);
+    rec.y = (int32_t)v[kWalk + 0];
+    rec.z = (int32_t)v[kWalk + 1];
+    rec.w = (int32_t)v[kWalk + 2];
+    st_node(d.node + cslot, rec);
+    put_equation(W, S, lane, mk_agent(cslot), x);
+    if (S.np) {  // the walker's next pair
+      S.fwd = true;
+      S.ra = rec;
+      S.rb = rp;
     }
   }
-  __syncwarp();
-  S.ac = __shfl_sync(kFull, ac, src);
-  S.vc = __shfl_sync(kFull, vc, src);
-  const long long dls = __shfl_sync(kFull, dl, src);
-  if (lane == 0) live += dls;
-  return valid ? np : 0u;
+#pragma unroll
+  for (int p = 0; p < 3; p++)
+    if (C.js[p] >= 0) put_equation(W, S, lane, r0[p], h0[p]);
 }
 
-// The warp's stacks hold the slots of one interaction of rule I.
-template <class Rules, int I>
-__device__ __forceinline__ bool lone_slots(const WarpStacks& S) {
-  constexpr uint32_t NN = Rules::kT[I].n_new;
-  return S.ac >= (int)(NN > 2 ? NN - 2 : 0) && S.vc >= (int)Rules::kT[I].n_fresh;
-}
-
-constexpr int kSpecialisedMaxNew = 2;
-// At most this many rules get their own code (the first in rule-table
-// order): every one adds to the run-time compile (up to about a second each:
-// a rule set of 64 rules compiles in about 33 s, once) and to the kernel's
-// code.
-constexpr int kSpecialisedMaxRules = 32;
-// Bit I set: rule I has its own code.
-template <class Rules>
-__host__ __device__ constexpr unsigned long long spec_mask() {
-  unsigned long long m = 0;
-  int k = 0;
-  for (int i = 0; i < Rules::kN && k < kSpecialisedMaxRules; i++)
-    if (Rules::kT[i].n_new <= kSpecialisedMaxNew) {
-      m |= 1ull << i;
-      k++;
+// A run of a rule that leaves its partners as they are (chain_passes): the
+// walker only has to find where the list ends, so the loop is a walk: along
+// neighbouring slots (numerals as they were loaded, copies as they were
+// allocated) kBlock partners at a time, their loads in flight together and
+// used as far as the list really goes through them; else one by one.  A
+// record loaded before the list was seen to lead to it is as good as one
+// loaded after: an agent that a record already reached names directly is
+// owned by this lane, was written before that record was published and does
+// not change.  What bounds it: one L2 round trip (337 ns) per block, partner
+// or name, so a turn of the loop issues whatever each lane waits for at once.
+// A chain of 20 891 Add: 26.2 ms with an interaction at a time, 6.9 ms in
+// run_rule, 2.3 ms here (0.11 us each); 4096 short sums 0.66 -> 0.13 ms.
+// Blocks of 4 against 8 and 16: 2048 Mul nets 4.4 / 5.1 / 5.8 ms,
+// Fibonacci(20..25) 26.6 / 27.3 / 29.5 ms, the chain 2.3 / 2.1 / 1.7 ms.
+template <bool kTrack, class Rules, int I, class WM>
+__device__ __forceinline__ void pass_rule(const Dev& d, WM& W, Lane& L, int lane, uint32_t a, uint32_t b,
+                                          const int4& ra, const int4& rb, uint32_t net, uint32_t lim, Step& S) {
+  constexpr Template R = Rules::kT[I];
+  constexpr ChainInfo C = chain_info(R);
+  constexpr int kPort = C.e % 3;                                // the partner's port the walker goes on to
+  constexpr int kOut = C.js[0] >= 0 ? 0 : C.js[1] >= 0 ? 1 : 2;  // the walker's port of the output stream
+  constexpr uint32_t kLabel = R.lhs[1 - C.cs];
+  constexpr bool kNarrow = chain_arity(R, 1 - C.cs) == 1;       // head and one port hold a whole partner
+  constexpr uint32_t kBlock = 4;
+  const uint32_t cslot = C.cs == 0 ? a : b;
+  const uint32_t first = C.cs == 0 ? b : a;
+  const uint32_t cap = (uint32_t)d.cap_agents;
+  uint32_t cur = first;
+  int4 rc = C.cs == 0 ? rb : ra;  // the partner the walker is at, and its record
+  uint32_t x = get_aux(rc, kPort), steps = 1;
+  int end = 0;  // the walker has come to an agent of another label: 1: its record is nb, 2: the record's first half
+  int4 nb = make_int4(0, 0, 0, 0);
+  for (uint32_t guard = 0;; guard++) {
+    // one round trip for every lane of the warp, whatever it waits for: a
+    // name, or the next partners
+    const uint32_t at = idx_of(x);
+    const bool name = is_var(x);
+    if (name ? at >= d.cap_vars || guard > 2 * lim : !is_agent(x) || at >= cap || steps >= lim) break;
+    // neighbouring slots: the whole block
+    const uint32_t dir = at - cur;
+    const bool block = !name && ((dir == 1u && at + kBlock <= cap) || (dir == ~0u && at + 1 >= kBlock));
+    uint32_t old = kEmpty;
+    int4 w[kBlock];
+    if (name) old = ld_volatile(d.var + at);
+    else w[0] = ld_partner<kNarrow>(d.node + at);
+    if (block) {
+#pragma unroll
+      for (int j = 1; j < (int)kBlock; j++) w[j] = ld_partner<kNarrow>(d.node + (at + (uint32_t)j * dir));
     }
-  return m;
+    if (name) {
+      // one whose other occurrence has arrived: this one is the second (the
+      // slot is finished, nobody else refers to it), so the walker goes on
+      // without being published; an empty one ends the run
+      if (old == kEmpty) break;
+      release_name<kTrack>(d, W, L, lane, at);
+      x = old;
+      if (is_agent(x)) {
+        set_aux(rc, kPort, x);
+        st_node(d.node + cur, rc);
+      }
+      continue;
+    }
+    if (((uint32_t)w[0].x & 0xFFu) != kLabel) {
+      end = kNarrow ? 2 : 1;
+      nb = w[0];
+      break;
+    }
+    steps++;
+    cur = at;
+    rc = w[0];
+    x = get_aux(rc, kPort);
+    if (block) {
+      bool on = true, other = false;
+#pragma unroll
+      for (int j = 1; j < (int)kBlock; j++) {
+        on = on && x == mk_agent(at + (uint32_t)j * dir);
+        if (on && ((uint32_t)w[j].x & 0xFFu) != kLabel) {
+          on = false;
+          other = true;
+          nb = w[j];
+        }
+        if (on) {
+          steps++;
+          cur = at + (uint32_t)j * dir;
+          x = get_aux(w[j], kPort);
+          rc = w[j];
+        }
+      }
+      if (other) {
+        end = kNarrow ? 2 : 1;
+        break;
+      }
+    }
+  }
+  const int4& rw = C.cs == 0 ? ra : rb;
+  const uint32_t r0 = get_aux(rw, kOut);
+  S.steps = steps;
+  bool ended = false;
+  if (end) {
+    const uint32_t c[3] = {get_aux(rw, 0), get_aux(rw, 1), get_aux(rw, 2)};
+    const uint32_t hs[3] = {cur, cur, cur};
+    int4 hr[3] = {rc, rc, rc};
+    ended = end_run<kTrack, Rules, I, kNarrow>(d, W, L, lane, net, cslot, c, idx_of(x), nb, hs, hr, S);
+  }
+  if (!ended) {
+    // the last partner's and the walker's port get a name
+    const uint32_t w = mk_var(take_name<kTrack>(d, W, L, lane, net));
+    set_aux(rc, kPort, w);
+    st_node(d.node + cur, rc);
+    S.ra = rw;
+    set_aux(S.ra, kOut, w);
+    st_node(d.node + cslot, S.ra);
+    put_equation(W, S, lane, mk_agent(cslot), x);
+    S.fwd = S.np != 0;  // the walker's next pair
+    S.have_b = end == 1;
+    S.rb = nb;
+  }
+  put_equation(W, S, lane, r0, mk_agent(first));
 }
-template <class Rules, int I>
-__host__ __device__ constexpr bool specialised() {
-  return I < Rules::kN && ((spec_mask<Rules>() >> I) & 1ull);
+
+// The templates of the rules with their own code (which may hold reduced
+// pairs) in place of the loaded ones.
+template <class Rules, int I = 0>
+__device__ __forceinline__ void spec_templates(AsyncTpl* tmpl) {
+  if constexpr (I < Rules::kN && I < kSpecialisedMaxRules) {
+    constexpr Template R = Rules::kT[I];
+    constexpr uint32_t kIn = Rules::kMore[I][0] | (Rules::kMore[I][1] << 8) | (Rules::kMore[I][2] << 16);
+    if (threadIdx.x == I) tmpl[I] = pack_template(R, kIn);
+    spec_templates<Rules, I + 1>(tmpl);
+  }
 }
-#define INET_UNI_CASE(I)                                                                                   \
-  case I:                                                                                                  \
-    if constexpr (specialised<Rules, I>()) {                                                               \
-      if constexpr (chain_rule<Rules, I>()) {                                                              \
-        if (lone && lone_slots<Rules, I>(S))                                                               \
-          return lone_chain<kTrack, Rules, I>(d, tab, hist, W, S, valid, a, b, ra, rb, net, live);         \
-      }                                                                                                    \
-      return uni_interact<kTrack, Rules, I>(d, tab, hist, W, S, valid, vmask, a, b, ra, rb, net, live, quiet); \
-    }                                                                                                      \
+static_assert(kSpecialisedMaxRules <= 32, "one thread of the smallest block per rule");
+
+// Bit I set: rule I repeats itself along lists.
+template <class Rules, int I = 0>
+__device__ constexpr uint32_t run_mask() {
+  if constexpr (I < Rules::kN && I < kSpecialisedMaxRules)
+    return (chain_info(Rules::kT[I]).ok ? 1u << I : 0u) | run_mask<Rules, I + 1>();
+  else return 0u;
+}
+
+// One interaction of a rule read from shared memory.  The general kernel
+// keeps the values in a table; a specialised one, where few lanes come here,
+// finds each where it is: the arguments in
+// registers, the new slots on top of the lane's columns.
+template <bool kTrack, class WM>
+__device__ __forceinline__ void interpret(const Dev& d, WM& W, Lane& L, int lane, const AsyncTpl& T, uint32_t a,
+                                          uint32_t b, const int4& ra, const int4& rb, uint32_t net, Step& S) {
+  const uint32_t hdr = T.hdr;
+  const uint32_t n_new = hdr & 0xFFu, n_fresh = (hdr >> 8) & 0xFFu, n_link = (hdr >> 16) & 0xFFu;
+  const int ta = L.na, tv = L.nv;
+  auto value = [&](uint32_t c) -> uint32_t {
+    if constexpr (WM::kHasTable) {
+      return W.vals[c][lane];
+    } else {
+      if (c < (uint32_t)kValNew) {
+        const uint32_t q = c < 3 ? c : c - 3;
+        return get_aux(c < 3 ? ra : rb, (int)q);
+      }
+      if (c < (uint32_t)kValFresh) {
+        const int j = (int)c - kValNew;
+        return mk_agent(j == 0 ? a : j == 1 ? b : W.ares[ta - 1 - (j - 2)][lane]);
+      }
+      return mk_var(W.vres[tv - 1 - ((int)c - kValFresh)][lane]);
+    }
+  };
+  auto port = [&](uint32_t c) -> int32_t { return c == kValNone ? 0 : (int32_t)value(c); };
+  if constexpr (WM::kHasTable) {
+    W.vals[kValExt + 0][lane] = (uint32_t)ra.y;
+    W.vals[kValExt + 1][lane] = (uint32_t)ra.z;
+    W.vals[kValExt + 2][lane] = (uint32_t)ra.w;
+    W.vals[kValExt + 3][lane] = (uint32_t)rb.y;
+    W.vals[kValExt + 4][lane] = (uint32_t)rb.z;
+    W.vals[kValExt + 5][lane] = (uint32_t)rb.w;
+    if (n_new > 0) W.vals[kValNew + 0][lane] = mk_agent(a);
+    if (n_new > 1) W.vals[kValNew + 1][lane] = mk_agent(b);
+  }
+  for (uint32_t j = 2; j < n_new; j++) {
+    const uint32_t sl = take_agent(W, L, lane);
+    if constexpr (WM::kHasTable) W.vals[kValNew + j][lane] = mk_agent(sl);
+  }
+  for (uint32_t f = 0; f < n_fresh; f++) {
+    const uint32_t x = take_name<kTrack>(d, W, L, lane, net);
+    if constexpr (WM::kHasTable) W.vals[kValFresh + f][lane] = mk_var(x);
+  }
+  for (uint32_t j = 0; j < n_new; j++) {
+    const uint32_t w = T.agent[j];
+    int4 rec;
+    rec.x = (int32_t)((net << 8) | (w & 0xFFu));
+    rec.y = port((w >> 8) & 0xFFu);
+    rec.z = port((w >> 16) & 0xFFu);
+    rec.w = port(w >> 24);
+    st_node(d.node + idx_of(value(kValNew + j)), rec);
+  }
+  S.steps = 1;
+  for (uint32_t k = 0; k < n_link; k++) {
+    const uint32_t lk = T.link[k];
+    put_equation(W, S, lane, value(lk & 0xFFu), value(lk >> 8));
+  }
+  if (n_new == 0) put_agent<kTrack>(d, W, L, lane, a);
+  if (n_new < 2) put_agent<kTrack>(d, W, L, lane, b);
+  L.live += (long long)n_new - 2;
+}
+
+template <bool kTrack, class Rules, int I, class WM>
+__device__ __forceinline__ void spec_rule(const Dev& d, WM& W, Lane& L, int lane, uint32_t a, uint32_t b,
+                                          const int4& ra, const int4& rb, uint32_t net, uint32_t lim,
+                                          Step& S) {
+  if constexpr (I < Rules::kN && I < kSpecialisedMaxRules) {
+    if constexpr (chain_passes(Rules::kT[I], chain_info(Rules::kT[I])))
+      pass_rule<kTrack, Rules, I>(d, W, L, lane, a, b, ra, rb, net, lim, S);
+    else if constexpr (chain_info(Rules::kT[I]).ok) run_rule<kTrack, Rules, I>(d, W, L, lane, a, b, ra, rb, net, lim, S);
+    else one_step<kTrack, Rules, I>(d, W, L, lane, a, b, ra, rb, net, S);
+  }
+}
+#define INET_SPEC_CASE(I)                                                             \
+  case I:                                                                             \
+    spec_rule<kTrack, Rules, I>(d, W, L, lane, a, b, ra, rb, net, lim, S);             \
     break;
 
-// One interaction per lane whose `valid` is set (warp-collective).  The new
-// active pairs are left in W.out[0..return)[lane]; a pair that cannot be
-// reduced (no rule, corrupt state) is dropped and returns 0.  Lane 0's
-// `live` collects the change of live agents.  With a specialised rule set,
-// a warp whose lanes all reduce the same rule takes that rule's own code;
-// any other warp (and the general kernel always) interprets the templates
-// in shared memory.
-template <bool kTrack, class Rules>
-__device__ __forceinline__ uint32_t async_interact(const Dev& d, const AsyncTpl* tmpl, const int16_t* tab,
-                                                   uint32_t* hist, WarpMem& W, WarpStacks& S, bool valid,
-                                                   uint32_t a, uint32_t b, long long& live, bool pre,
-                                                   int4 pra, int4 prb, bool lone, bool quiet) {
+// One step of each lane whose `valid` is set: an interaction, or a run of
+// them (warp-collective).  The new active pairs are left in
+// W.out[0..S.np)[lane]; a pair that cannot be reduced (no rule, corrupt
+// state) is dropped.
+template <bool kTrack, class Rules, class WM>
+__device__ __forceinline__ void async_interact(const Dev& d, const AsyncTpl* tmpl, const int16_t* tab,
+                                               uint32_t* hist, WM& W, Lane& L, bool valid, uint32_t a,
+                                               uint32_t b, bool pre, int4 ra, int4 rb, Step& S) {
   const int lane = threadIdx.x & 31;
-  Ctrl* c = d.ctrl;
   uint32_t net = 0, ti = 0;
-  int4 ra = make_int4(0, 0, 0, 0), rb = ra;
+  S.np = S.ne = S.steps = 0;
+  S.fwd = S.have_b = false;
+  S.fin = -1;
   if (valid && (a >= d.cap_agents || b >= d.cap_agents)) {
-    set_error(c, INET_ERR_STATE, 2);
+    report(d, INET_ERR_STATE, 2);
     valid = false;
   }
   if (valid) {
-    if (pre) {
-      ra = pra;
-      rb = prb;
-    } else {
+    if (!pre) {
       ra = ld_node(d.node + a);
       rb = ld_node(d.node + b);
     }
@@ -796,12 +1172,12 @@ __device__ __forceinline__ uint32_t async_interact(const Dev& d, const AsyncTpl*
     const int e = (la < d.n_labels && lb < d.n_labels) ? tab[la * d.n_labels + lb] : -1;
     net = (uint32_t)ra.x >> 8;
     if (net >= d.max_nets) {
-      set_error(c, INET_ERR_STATE, 3);
+      report(d, INET_ERR_STATE, 3);
       valid = false;
     } else if (e < 0) {
       valid = false;
       atomicCAS(d.netstat + net, 0, INET_ERR_NO_RULE);
-      set_error(c, INET_ERR_NO_RULE, net);
+      report(d, INET_ERR_NO_RULE, net);
       atomicAdd(d.netctr + net, (unsigned long long)(-(1ll << kNetPairShift)));
     } else {
       if (e & 1) {
@@ -811,107 +1187,73 @@ __device__ __forceinline__ uint32_t async_interact(const Dev& d, const AsyncTpl*
       ti = (uint32_t)e >> 1;
     }
   }
+  const uint32_t hdr = valid ? tmpl[ti].hdr : 0u;
+  const uint32_t n_new = hdr & 0xFFu, need_a = n_new > 2 ? n_new - 2 : 0u, need_v = (hdr >> 8) & 0xFFu;
+  const unsigned lack = __ballot_sync(kFull, (uint32_t)L.na < need_a || (uint32_t)L.nv < need_v);
+  if (lack) {
+    bool runs = false;
+    if constexpr (Rules::kN > 0) runs = (run_mask<Rules>() >> (ti & 31u)) & 1u;
+    if (!refill(d, W, L, runs, need_a, need_v, lane)) return;  // fatal: the loop stops
+  }
+  // a run keeps the warp's other lanes waiting, and what waits for its output
+  uint32_t lim = 1;
   if constexpr (Rules::kN > 0) {
-    const unsigned vmask = __ballot_sync(kFull, valid);
-    const uint32_t lead = __shfl_sync(kFull, ti, vmask ? __ffs(vmask) - 1 : 0);
-    if (vmask && ((spec_mask<Rules>() >> lead) & 1ull) && __all_sync(kFull, !valid || ti == lead)) {
-      switch (lead) {
-        INET_UNI_CASE(0) INET_UNI_CASE(1) INET_UNI_CASE(2) INET_UNI_CASE(3) INET_UNI_CASE(4) INET_UNI_CASE(5)
-        INET_UNI_CASE(6) INET_UNI_CASE(7) INET_UNI_CASE(8) INET_UNI_CASE(9) INET_UNI_CASE(10) INET_UNI_CASE(11)
-        INET_UNI_CASE(12) INET_UNI_CASE(13) INET_UNI_CASE(14) INET_UNI_CASE(15) INET_UNI_CASE(16) INET_UNI_CASE(17)
-        INET_UNI_CASE(18) INET_UNI_CASE(19) INET_UNI_CASE(20) INET_UNI_CASE(21) INET_UNI_CASE(22) INET_UNI_CASE(23)
-        INET_UNI_CASE(24) INET_UNI_CASE(25) INET_UNI_CASE(26) INET_UNI_CASE(27) INET_UNI_CASE(28) INET_UNI_CASE(29)
-        INET_UNI_CASE(30) INET_UNI_CASE(31) INET_UNI_CASE(32) INET_UNI_CASE(33) INET_UNI_CASE(34) INET_UNI_CASE(35)
-        INET_UNI_CASE(36) INET_UNI_CASE(37) INET_UNI_CASE(38) INET_UNI_CASE(39) INET_UNI_CASE(40) INET_UNI_CASE(41)
-        INET_UNI_CASE(42) INET_UNI_CASE(43) INET_UNI_CASE(44) INET_UNI_CASE(45) INET_UNI_CASE(46) INET_UNI_CASE(47)
-        INET_UNI_CASE(48) INET_UNI_CASE(49) INET_UNI_CASE(50) INET_UNI_CASE(51) INET_UNI_CASE(52) INET_UNI_CASE(53)
-        INET_UNI_CASE(54) INET_UNI_CASE(55) INET_UNI_CASE(56) INET_UNI_CASE(57) INET_UNI_CASE(58) INET_UNI_CASE(59)
-        INET_UNI_CASE(60) INET_UNI_CASE(61) INET_UNI_CASE(62) INET_UNI_CASE(63)
-        default: break;
-      }
-    }
+    const bool one = valid && !(ti < 32 && ((run_mask<Rules>() >> (ti & 31u)) & 1u));
+    const int all = __popc(__ballot_sync(kFull, valid)), ones = __popc(__ballot_sync(kFull, one));
+    lim = all == 1 ? kRunLone : 2 * ones > all ? kRunMixed : kRunMany;
   }
-  static_assert(INET_MAX_RULES == 64, "one case per rule");
-  const AsyncTpl& T = tmpl[ti];
-  const uint32_t hdr = valid ? T.hdr : 0u;
-  const uint32_t n_new = hdr & 0xFFu, n_fresh = (hdr >> 8) & 0xFFu, n_link = (hdr >> 16) & 0xFFu;
-  const uint32_t need_a = n_new > 2 ? n_new - 2 : 0u;
-  const uint32_t free_a = valid && n_new < 2 ? 2 - n_new : 0u;
-  // a3: offsets of this lane among the warp's needs (10 bits per field;
-  // a warp needs at most 32 x 8)
-  const uint32_t packed = need_a | (n_fresh << 10) | (free_a << 20);
-  uint32_t inc = packed;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const uint32_t t = __shfl_up_sync(kFull, inc, o);
-    if (lane >= o) inc += t;
-  }
-  const uint32_t tot = __shfl_sync(kFull, inc, 31), ex = inc - packed;
-  const uint32_t Ka = tot & 1023u, Kv = (tot >> 10) & 1023u, Fa = tot >> 20;
-  const uint32_t oa = ex & 1023u, ov = (ex >> 10) & 1023u, of = ex >> 20;
-  PopPlan P;
-  if (!warp_pop(d, S, Ka, Kv, lane, P)) return 0u;
-  if (lane == 0) live += (long long)Ka - (long long)Fa;
   if (valid) {
-    W.vals[kValExt + 0][lane] = (uint32_t)ra.y;
-    W.vals[kValExt + 1][lane] = (uint32_t)ra.z;
-    W.vals[kValExt + 2][lane] = (uint32_t)ra.w;
-    W.vals[kValExt + 3][lane] = (uint32_t)rb.y;
-    W.vals[kValExt + 4][lane] = (uint32_t)rb.z;
-    W.vals[kValExt + 5][lane] = (uint32_t)rb.w;
-    bool in_range = true;
-    if (n_new > 0) W.vals[kValNew + 0][lane] = mk_agent(a);
-    if (n_new > 1) W.vals[kValNew + 1][lane] = mk_agent(b);
-    for (uint32_t j = 2; j < n_new; j++) {
-      const uint32_t sl = plan_agent(d, W, P, oa + j - 2);
-      if (sl >= d.cap_agents) in_range = false;
-      W.vals[kValNew + j][lane] = mk_agent(sl);
-    }
-    for (uint32_t v = 0; v < n_fresh; v++) {
-      const uint32_t x = plan_var(d, W, P, ov + v);
-      if (x >= d.cap_vars) {
-        in_range = false;
-      } else {
-        __stcg(d.var + x, kEmpty);  // a fresh name starts empty; published by this lane's fence
-        if constexpr (kTrack) __stcg(d.vown + x, net);
+    if constexpr (Rules::kN == 0) {
+      interpret<kTrack>(d, W, L, lane, tmpl[ti], a, b, ra, rb, net, S);
+    } else {
+      switch (ti) {
+        INET_SPEC_CASE(0) INET_SPEC_CASE(1) INET_SPEC_CASE(2) INET_SPEC_CASE(3) INET_SPEC_CASE(4) INET_SPEC_CASE(5)
+        INET_SPEC_CASE(6) INET_SPEC_CASE(7) INET_SPEC_CASE(8) INET_SPEC_CASE(9) INET_SPEC_CASE(10) INET_SPEC_CASE(11)
+        INET_SPEC_CASE(12) INET_SPEC_CASE(13) INET_SPEC_CASE(14) INET_SPEC_CASE(15) INET_SPEC_CASE(16)
+        INET_SPEC_CASE(17) INET_SPEC_CASE(18) INET_SPEC_CASE(19) INET_SPEC_CASE(20) INET_SPEC_CASE(21)
+        INET_SPEC_CASE(22) INET_SPEC_CASE(23) INET_SPEC_CASE(24) INET_SPEC_CASE(25) INET_SPEC_CASE(26)
+        INET_SPEC_CASE(27) INET_SPEC_CASE(28) INET_SPEC_CASE(29) INET_SPEC_CASE(30) INET_SPEC_CASE(31)
+        default:
+          if constexpr (Rules::kN > kSpecialisedMaxRules)
+            interpret<kTrack>(d, W, L, lane, tmpl[ti], a, b, ra, rb, net, S);
+          break;
       }
-      W.vals[kValFresh + v][lane] = mk_var(x);
-    }
-    if (!in_range) {
-      set_error(c, INET_ERR_STATE, 4);
-      valid = false;
+      static_assert(kSpecialisedMaxRules == 32, "one case per rule with its own code");
     }
   }
-  __syncwarp();  // every taken stack entry has been read
-  warp_settle<kTrack>(d, W, S, P, Fa, free_a, of, n_new == 0, a, b, lane);
-  // a2: the new agents' records
-  uint32_t np = 0;
+  if (__any_sync(kFull, S.ne != 0)) {
+    __threadfence();
+    if (S.ne) link_lane<kTrack>(d, W, L, S, lane);
+  }
   if (valid) {
-    const uint32_t head_net = net << 8;
-    for (uint32_t j = 0; j < n_new; j++) {
-      const uint32_t w = T.agent[j];
-      int4 rec;
-      rec.x = (int32_t)(head_net | (w & 0xFFu));
-      rec.y = port_val(W, (w >> 8) & 0xFFu, lane);
-      rec.z = port_val(W, (w >> 16) & 0xFFu, lane);
-      rec.w = port_val(W, w >> 24, lane);
-      st_node(d.node + idx_of(W.vals[kValNew + j][lane]), rec);
+    // per-net counters (interactions and the change of pending pairs) and
+    // the rule histogram: one fire-and-forget atomic each; with kTrack the
+    // net's live agents too (its quota is checked between launches)
+    const uint32_t in = tmpl[ti].inside, n_in = in & 0xFFu;
+    uint32_t ints = S.steps * (1 + n_in);
+    long long dlive = ((long long)n_new - 2) * (long long)S.steps;
+    atomicAdd(&hist[hdr >> 24], S.steps);
+    if (n_in > 0) atomicAdd(&hist[(in >> 8) & 0xFFu], S.steps);
+    if (n_in > 1) atomicAdd(&hist[(in >> 16) & 0xFFu], S.steps);
+    if (Rules::kN > 0 && S.fin >= 0) {
+      const uint32_t fh = tmpl[S.fin].hdr, fi = tmpl[S.fin].inside, f_in = fi & 0xFFu;
+      ints += 1 + f_in;
+      dlive += (long long)(fh & 0xFFu) - 2;
+      atomicAdd(&hist[fh >> 24], 1u);
+      if (f_in > 0) atomicAdd(&hist[(fi >> 8) & 0xFFu], 1u);
+      if (f_in > 1) atomicAdd(&hist[(fi >> 16) & 0xFFu], 1u);
     }
-    // a4: link
-    if (n_link)
-      np = link_lane<kTrack, -1>(d, W, n_link, [&](uint32_t k, int s) {
-        const uint32_t lk = T.link[k];
-        return W.vals[s ? lk >> 8 : lk & 0xFFu][lane];
-      }, lane);
+    atomicAdd(d.netctr + net, (unsigned long long)ints + ((unsigned long long)((long long)S.np - 1) << kNetPairShift));
+    if constexpr (kTrack) {
+      if (dlive) atomicAdd(reinterpret_cast<unsigned long long*>(d.netlive + net), (unsigned long long)dlive);
+    }
   }
-  flush_vstage(d, W, S, lane);
-  if (valid) count_interaction<kTrack>(d, hist, net, hdr >> 24, np, n_new);
-  return valid ? np : 0u;
+  __syncwarp();
 }
-#undef INET_UNI_CASE
+#undef INET_SPEC_CASE
 
 // Writes a pair back to the exit frontier (other buffer).
-__device__ __forceinline__ void exit_pair(const Dev& d, Pair p) {
+__device__ __noinline__ void exit_pair(const Dev& d, Pair p) {
   const uint32_t k = atomicAdd(&d.ctrl->aexit, 1u);
   if (k < d.cap_pairs) {
     __stcg(reinterpret_cast<unsigned long long*>(d.front[d.qcur ^ 1u] + k), *reinterpret_cast<unsigned long long*>(&p));
@@ -941,7 +1283,7 @@ __device__ __forceinline__ void poll_ticket(const Dev& d, const Pair* Q, bool& h
 
 // Bounded wait for ticket t's pair (when no producer runs any more);
 // returns false on timeout.
-__device__ __forceinline__ bool wait_ticket(const Dev& d, const Pair* Q, unsigned long long t, Pair* out) {
+__device__ __noinline__ bool wait_ticket(const Dev& d, const Pair* Q, unsigned long long t, Pair* out) {
   const unsigned long long s = t % d.cap_pairs;
   const unsigned long long t0 = globaltimer();
   for (uint32_t spin = 0;; spin++) {
@@ -964,11 +1306,15 @@ __global__ void __launch_bounds__(256, 2) k_async(Dev d) {
   size_t off = 0;
   auto take = [&](size_t n) { off = (off + 15) / 16 * 16; unsigned char* p = smem_raw + off; off += n; return p; };
   AsyncTpl* tmpl = reinterpret_cast<AsyncTpl*>(take(sizeof(AsyncTpl) * (d.n_tmpl ? d.n_tmpl : 1)));
-  WarpMem* wm = reinterpret_cast<WarpMem*>(take(sizeof(WarpMem) * (blockDim.x / 32)));
+  using WM = WarpMem<Rules::kN == 0>;
+  WM* wm = reinterpret_cast<WM*>(take(sizeof(WM) * (blockDim.x / 32)));
   uint32_t* hist = reinterpret_cast<uint32_t*>(take(sizeof(uint32_t) * INET_MAX_RULES));
   int16_t* tab = reinterpret_cast<int16_t*>(take(sizeof(int16_t) * d.n_labels * d.n_labels));
+#pragma unroll 1
   for (uint32_t i = threadIdx.x; i < d.n_tmpl; i += blockDim.x) tmpl[i] = pack_template(d.tmpl[i]);
+#pragma unroll 1
   for (uint32_t i = threadIdx.x; i < d.n_labels * d.n_labels; i += blockDim.x) tab[i] = d.table[i];
+#pragma unroll 1
   for (uint32_t i = threadIdx.x; i < INET_MAX_RULES; i += blockDim.x) hist[i] = 0;
   if constexpr (Rules::kN > 0) {
     // a specialised kernel runs only on the rule set it was built for (the
@@ -980,10 +1326,14 @@ __global__ void __launch_bounds__(256, 2) k_async(Dev d) {
     }
   }
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  WarpMem& W = wm[wid];
-  if (lane == 0) W.vstage_n = 0;
-  WarpStacks S{0, 0};
+  WM& W = wm[wid];
+  if (lane == 0) W.an = W.vn = 0;
+  Lane L{0, 0, 0};
   __syncthreads();
+  if constexpr (Rules::kN > 0) {
+    spec_templates<Rules>(tmpl);
+    __syncthreads();
+  }
   Ctrl* c = d.ctrl;
   Pair* Q = d.front[d.qcur];
   const unsigned long long cap = d.cap_pairs;
@@ -991,11 +1341,10 @@ __global__ void __launch_bounds__(256, 2) k_async(Dev d) {
   bool have = false;
   uint32_t pa = 0, pb = 0;
   unsigned long long ticket = kNoTicket, tslot = 0;
-  long long live = 0;
-  uint32_t nap = 0;
+  uint32_t nap = 0, flag = 0;
+  unsigned long long qh = 0, qt = 0;
   bool stop = false, finished = false, check_now = false;
   bool pre = false;
-  bool qseen = false;  // the queue held pairs when this warp last looked
   int4 pra = make_int4(0, 0, 0, 0), prb = pra;
   unsigned long long t_start = 0;
   if (lane == 0) {
@@ -1004,13 +1353,17 @@ __global__ void __launch_bounds__(256, 2) k_async(Dev d) {
     t_start = ld_volatile64(&c->slice_t0);
   }
   for (uint32_t it = 0;; it++) {
-    // stop / slice checks every 16 iterations, and when a napping warp's
-    // clock says the time slice is over
+    // stop / slice checks every 16 iterations (on flags loaded during the
+    // iteration before), and when a napping warp's clock says the time
+    // slice is over
     if ((it & 15) == 15 || check_now) {
+      if (check_now) {
+        if (lane == 1) flag = ld_volatile(&c->astop);
+        if (lane == 2) flag = ld_volatile((const uint32_t*)&c->fatal);
+      }
       check_now = false;
-      uint32_t st = 0;
+      uint32_t st = __any_sync(kFull, flag != 0) ? 1u : 0u;
       if (lane == 0) {
-        st = ld_volatile(&c->astop) | (ld_volatile((const uint32_t*)&c->fatal) ? 1u : 0u);
         if (!st && globaltimer() - t_start > d.slice_ns) {
           c->astop = 1;
           c->hit_slice = 1;
@@ -1034,12 +1387,11 @@ __global__ void __launch_bounds__(256, 2) k_async(Dev d) {
     const unsigned busy = __ballot_sync(kFull, have);
     if (want && (!busy || (it & 7) == 0)) {
       unsigned long long base = 0;
-      uint32_t k = 0, qs = 0;
+      uint32_t k = 0;
       if (lane == 0) {
-        unsigned long long qh, qt;
-        asm volatile("ld.volatile.global.v2.u64 {%0, %1}, [%2];" : "=l"(qh), "=l"(qt) : "l"(&c->q_head) : "memory");
+        // a busy warp looks at what it loaded during the iteration before
+        if (!busy) asm volatile("ld.volatile.global.v2.u64 {%0, %1}, [%2];" : "=l"(qh), "=l"(qt) : "l"(&c->q_head) : "memory");
         const unsigned long long backlog = qt > qh ? qt - qh : 0ull;
-        qs = backlog ? 1u : 0u;
         const bool deep = backlog > total_warps;
         if (backlog && (!busy || deep)) {
           k = (uint32_t)min(min((unsigned long long)__popc(want), backlog), deep ? 32ull : 1ull);
@@ -1047,7 +1399,6 @@ __global__ void __launch_bounds__(256, 2) k_async(Dev d) {
         }
       }
       k = __shfl_sync(kFull, k, 0);
-      qseen = __shfl_sync(kFull, qs, 0) != 0;
       if (k) {
         unsigned long long bm = 0;
         if (lane == 0) bm = base % cap;
@@ -1067,6 +1418,8 @@ __global__ void __launch_bounds__(256, 2) k_async(Dev d) {
       // idle: the loop is over when no pair is left anywhere
       uint32_t fin = 0;
       if (lane == 0) fin = ld_volatile_s64(&c->inflight) == 0 ? 1u : 0u;
+      if (lane == 1) flag = ld_volatile(&c->astop);
+      if (lane == 2) flag = ld_volatile((const uint32_t*)&c->fatal);
       if (__shfl_sync(kFull, fin, 0)) {
         finished = true;
         break;
@@ -1081,32 +1434,33 @@ __global__ void __launch_bounds__(256, 2) k_async(Dev d) {
       {
         uint32_t late = 0;
         if (lane == 0) late = globaltimer() - t_start > d.slice_ns ? 1u : 0u;
-        check_now = __shfl_sync(kFull, late, 0) != 0;
+        check_now = __any_sync(kFull, late != 0 || flag != 0);
       }
       continue;
     }
     nap = 0;
-    // no lane waits for a ticket and the queue was empty when the warp last
-    // looked: chains may run without the warp's loop (queued work is left to
-    // the loop, whose idle lanes claim it); lone: one lane holds a pair
-    const bool quiet = !qseen && __ballot_sync(kFull, ticket != kNoTicket) == 0;
-    const bool lone = quiet && __popc(act) == 1;
-    const uint32_t np = async_interact<kTrack, Rules>(d, tmpl, tab, hist, W, S, have, pa, pb, live, pre, pra, prb,
-                                                      lone, quiet);
-    // keep the first new pair and start loading its records now, so the
-    // load overlaps the rest of this iteration
+    if ((it & 15) == 14) {
+      if (lane == 1) flag = ld_volatile(&c->astop);
+      if (lane == 2) flag = ld_volatile((const uint32_t*)&c->fatal);
+    }
+    const bool look = (it & 7) == 7;
+    if (look && lane == 0)
+      asm volatile("ld.volatile.global.v2.u64 {%0, %1}, [%2];" : "=l"(qh), "=l"(qt) : "l"(&c->q_head) : "memory");
+    Step S;
+    async_interact<kTrack, Rules>(d, tmpl, tab, hist, W, L, have, pa, pb, pre, pra, prb, S);
+    const uint32_t np = S.np;
+    // keep the first new pair; the records the step hands on in registers
+    // need no load, the others are loaded below
     const bool had = have;
     have = np > 0;
-    pre = false;
+    bool lda = have && !S.fwd, ldb = have && (!S.fwd || !S.have_b);
+    pre = have;
     if (have) {
       const Pair p0 = W.out[0][lane];
       pa = p0.a;
       pb = p0.b;
-      if (pa < d.cap_agents && pb < d.cap_agents) {
-        pra = ld_node(d.node + pa);
-        prb = ld_node(d.node + pb);
-        pre = true;
-      }
+      pra = S.ra;
+      prb = S.rb;
     }
     const uint32_t extra = np > 1 ? np - 1 : 0u;
     // pairs in flight: each new pair beyond a lane's own next one joins
@@ -1123,20 +1477,21 @@ __global__ void __launch_bounds__(256, 2) k_async(Dev d) {
     // is held by a claimed ticket whenever it is still occupied: an
     // unclaimed one would put every later ticket, and so more than cap
     // pairs, in flight.
-    const long long grow = (long long)__reduce_add_sync(kFull, extra);
-    const long long shrink = -(long long)__reduce_add_sync(kFull, had && np == 0 ? 1u : 0u);
-    if (grow) {
+    const long long shrink = -(long long)__popc(__ballot_sync(kFull, had && np == 0));
+    unsigned more = __ballot_sync(kFull, extra != 0);
+    if (more) {
       // extra pairs go first to idle lanes of this warp (through shared
       // memory), the rest to the ticket queue
-      unsigned inc = extra;
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const unsigned t = __shfl_up_sync(kFull, inc, o);
-        if (lane >= o) inc += t;
+      // the lanes' first extra pairs, then their second ones, ...
+      unsigned totx = 0;
+#pragma unroll 1
+      for (uint32_t j = 0; more; j++) {
+        if (j < extra) W.xl[totx + __popc(more & lanemask_lt())] = W.out[1 + j][lane];
+        totx += __popc(more);
+        more = __ballot_sync(kFull, j + 1 < extra);
       }
-      const unsigned totx = __shfl_sync(kFull, inc, 31);
-      if (totx) {
-        for (uint32_t j = 0; j < extra; j++) W.xl[inc - extra + j] = W.out[1 + j][lane];
+      {
+        const long long grow = (long long)totx;
         const unsigned idle = __ballot_sync(kFull, !have && ticket == kNoTicket);
         const unsigned nidle = __popc(idle);
         __syncwarp();
@@ -1157,16 +1512,15 @@ __global__ void __launch_bounds__(256, 2) k_async(Dev d) {
             const Pair p = W.xl[r];
             pa = p.a;
             pb = p.b;
-            have = true;
-            if (pa < d.cap_agents && pb < d.cap_agents) {
-              pra = ld_node(d.node + pa);
-              prb = ld_node(d.node + pb);
-              pre = true;
-            }
+            have = pre = lda = ldb = true;
           }
         }
         const unsigned toq = totx - local;
         if (toq) {
+          // a step that left only agent-agent equations has not fenced: the
+          // records of every pair are published before the pair is
+          __threadfence();
+          __syncwarp();
           unsigned long long qb = 0, qm = 0;
           if (lane == 0) {
             qb = atomicAdd(&c->q_tail, (unsigned long long)toq);
@@ -1174,6 +1528,7 @@ __global__ void __launch_bounds__(256, 2) k_async(Dev d) {
           }
           qb = __shfl_sync(kFull, qb, 0);
           qm = __shfl_sync(kFull, qm, 0);
+#pragma unroll 1
           for (unsigned j0 = 0; j0 < toq; j0 += 32) {
             const unsigned j = j0 + (unsigned)lane;
             bool pend = j < toq;
@@ -1182,6 +1537,7 @@ __global__ void __launch_bounds__(256, 2) k_async(Dev d) {
             if (si >= cap) si %= cap;
             const Pair p = pend ? W.xl[local + j] : Pair{0, 0};
             const unsigned long long t0 = globaltimer();
+#pragma unroll 1
             for (uint32_t spin = 0;; spin++) {
               // written once the cell's previous pair (ticket tk - cap) is taken
               if (pend && ld_acquire64(d.qseq + si) == tk) {
@@ -1214,10 +1570,21 @@ __global__ void __launch_bounds__(256, 2) k_async(Dev d) {
       }
     }
     if (lane == 0 && shrink) atomicAdd(reinterpret_cast<unsigned long long*>(&c->inflight), (unsigned long long)shrink);
+    // one load for the lanes that keep a pair and the lanes handed one (two
+    // loads of the same registers would wait for each other), in flight
+    // during the next iteration's top
+    if (pa >= d.cap_agents || pb >= d.cap_agents) pre = lda = ldb = false;
+    if (lda) pra = ld_node(d.node + pa);
+    if (ldb) prb = ld_node(d.node + pb);
     __syncwarp();
   }
   // leaving: publish live agents; a stop drains every pair to the other buffer
-  if (lane == 0 && live) atomicAdd(reinterpret_cast<unsigned long long*>(&c->live), (unsigned long long)live);
+  {
+    long long live = L.live;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) live += __shfl_xor_sync(kFull, live, o);
+    if (lane == 0 && live) atomicAdd(reinterpret_cast<unsigned long long*>(&c->live), (unsigned long long)live);
+  }
   if (finished && !stop) {
     if (lane == 0) {
       __threadfence();
@@ -1265,6 +1632,7 @@ __global__ void __launch_bounds__(256, 2) k_async(Dev d) {
       // unclaimed tickets, shared among the warps
       const unsigned long long qh = ld_volatile64(&c->q_head);
       const uint32_t gw = blockIdx.x * (blockDim.x / 32) + (uint32_t)wid;
+#pragma unroll 1
       for (unsigned long long tk = qh + (unsigned long long)gw * 32 + lane; tk < qt;
            tk += (unsigned long long)total_warps * 32) {
         Pair p;
@@ -1273,31 +1641,48 @@ __global__ void __launch_bounds__(256, 2) k_async(Dev d) {
     }
   }
   // free slots known only to this warp go back to the rings (when owners are
-  // kept, marked free: a stack also holds slots fetched from the pools and
-  // never used, which may come from the bump pointer with stale contents)
+  // kept, marked free: some were fetched from the pools and never used, which
+  // may come from the bump pointer with stale contents)
   __syncwarp();
   {
+    const uint32_t ac = (uint32_t)min(W.an, kAStack), vc = (uint32_t)min(W.vn, kVStack);
+    uint32_t inc = (uint32_t)L.na | ((uint32_t)L.nv << 16);
+    const uint32_t own = inc;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t t = __shfl_up_sync(kFull, inc, o);
+      if (lane >= o) inc += t;
+    }
+    const uint32_t tot = __shfl_sync(kFull, inc, 31);
+    const uint32_t ta = ac + (tot & 0xFFFFu), tv = vc + (tot >> 16);
     unsigned long long ab = 0, vb = 0;
     if (lane == 0) {
-      if (S.ac) ab = atomicAdd(&c->a_tail, (unsigned long long)S.ac);
-      if (S.vc) vb = atomicAdd(&c->v_tail, (unsigned long long)S.vc);
+      if (ta) ab = atomicAdd(&c->a_tail, (unsigned long long)ta);
+      if (tv) vb = atomicAdd(&c->v_tail, (unsigned long long)tv);
     }
     ab = __shfl_sync(kFull, ab, 0);
     vb = __shfl_sync(kFull, vb, 0);
-    for (int j = lane; j < S.ac; j += 32) {
-      const uint32_t sl = W.astk[j];
+    auto give_agent = [&](unsigned long long at, uint32_t sl) {
       if constexpr (kTrack) {
         if (sl < d.cap_agents) __stcg(&d.node[sl].head, kFreeHead);
       }
-      __stcg(d.afree + (ab + j) % d.cap_agents, sl);
-    }
-    for (int j = lane; j < S.vc; j += 32) {
-      const uint32_t x = W.vstk[j];
+      __stcg(d.afree + at % d.cap_agents, sl);
+    };
+    auto give_name = [&](unsigned long long at, uint32_t x) {
       if constexpr (kTrack) {
         if (x < d.cap_vars) __stcg(d.vown + x, kNoNet);
       }
-      __stcg(d.vfree + (vb + j) % d.cap_vars, x);
-    }
+      __stcg(d.vfree + at % d.cap_vars, x);
+    };
+#pragma unroll 1
+    for (uint32_t j = (uint32_t)lane; j < ac; j += 32) give_agent(ab + j, W.astk[j]);
+#pragma unroll 1
+    for (uint32_t j = (uint32_t)lane; j < vc; j += 32) give_name(vb + j, W.vstk[j]);
+    const uint32_t ex = inc - own;
+#pragma unroll 1
+    for (int j = 0; j < L.na; j++) give_agent(ab + ac + (ex & 0xFFFFu) + (uint32_t)j, W.ares[j][lane]);
+#pragma unroll 1
+    for (int j = 0; j < L.nv; j++) give_name(vb + vc + (ex >> 16) + (uint32_t)j, W.vres[j][lane]);
   }
   __syncthreads();
   for (uint32_t i = threadIdx.x; i < d.n_tmpl; i += blockDim.x)

@@ -3,6 +3,7 @@
 #include "inet_jit.h"
 
 #include "inet.h"
+#include "inet_inside.h"
 
 #include <cuda_runtime.h>
 #include <dlfcn.h>
@@ -187,9 +188,19 @@ std::string jit_source(const Template* t, size_t n) {
   s += buf;
   snprintf(buf, sizeof buf, "  static constexpr unsigned long long kKey = %lluull;\n", (unsigned long long)rules_key(t, n));
   s += buf;
+  std::vector<Template> spec;
+  std::vector<std::vector<int>> more;
+  inside_rules(t, n, &spec, &more);
+  s += "  static constexpr unsigned char kMore[kN][3] = {";
+  for (size_t i = 0; i < n; i++) {
+    snprintf(buf, sizeof buf, "%s{%d, %d, %d}", i ? ", " : "", (int)more[i].size(), more[i].size() > 0 ? more[i][0] : 0,
+             more[i].size() > 1 ? more[i][1] : 0);
+    s += buf;
+  }
+  s += "};\n";
   s += "  static constexpr Template kT[kN] = {\n";
   for (size_t i = 0; i < n; i++) {
-    const Template& r = t[i];
+    const Template& r = spec[i];
     snprintf(buf, sizeof buf, "    {%u, %u, %u, %u, {", r.n_new, r.n_fresh, r.n_link, r.rule);
     s += buf;
     for (int j = 0; j < kMaxNew; j++) s += std::to_string(r.lab[j]) + (j + 1 < kMaxNew ? ", " : "}, {");

@@ -3,9 +3,9 @@
 // The general k_async interprets each rule's template (Sec. 2.2, ->int: the
 // agents of Theta, their ports and the equations of Theta') from shared
 // memory.  A rule set is fixed once loaded, so the same kernel can also be
-// compiled with the templates as constants (k_async<kTrack, Rules>): a warp
-// whose lanes all reduce one rule of at most two right-hand-side agents then
-// runs that rule's straight-line code, with the values in registers.  This
+// compiled with the templates as constants (k_async<kTrack, Rules>): each
+// lane then runs its rule's own code, with the values in registers, along
+// whole lists where the rule repeats itself.  This
 // unit generates that source for a rule set, compiles it at run time with
 // NVRTC (loaded with dlopen, so a missing NVRTC only turns the
 // specialisation off), loads the cubin and keeps it for the process; cubins
