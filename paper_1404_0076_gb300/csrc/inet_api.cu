@@ -32,7 +32,7 @@ namespace {
 
 constexpr uint32_t kTraceCap = 1u << 20;
 constexpr uint32_t kReadChunk = 1u << 16;  // nets per device walk of inet_readback_nats
-constexpr uint32_t kWalkMin = 256;         // S agents one thread walks before its net's agents are ranked
+constexpr uint32_t kWalkMin = 256;         // round trips of a net's walk before its agents are ranked
 constexpr uint64_t kDefaultAgents = 1ull << 22;
 constexpr uint64_t kDefaultVars = 1ull << 22;
 constexpr uint64_t kDefaultPairs = 1ull << 21;
@@ -570,8 +570,11 @@ inet_status ensure_net_counters(inet_ctx* ctx) {
 // quiescent for these nets (finished), so the slots below the host bump
 // counters hold every element of their lists.  No readback may be in
 // flight when the scratch grows.
+// `wait`: the caller waits for the values anyway, so the walks' outcome is
+// read first and the ranking (its launches alone take 0.15 ms) is queued only
+// when some walk ran out; else the ranking's kernels find that out themselves.
 inet_status read_nats_device(inet_ctx* ctx, cudaStream_t st, const uint32_t* droot, uint32_t m, int s_label,
-                             int z_label, unsigned long long* dval) {
+                             int z_label, unsigned long long* dval, bool wait) {
   const uint32_t na = (uint32_t)ctx->a_bump, nv = (uint32_t)ctx->v_bump;
   if (!ctx->jump_ctl) CK(cudaMalloc(&ctx->jump_ctl, sizeof(uint32_t) * kJumpCtl));
   if (na > ctx->jump_cap) {
@@ -591,11 +594,18 @@ inet_status read_nats_device(inet_ctx* ctx, cudaStream_t st, const uint32_t* dro
   uint8_t* mark = at<uint8_t>(ctx, ctx->lay.rbmark);
   CK(cudaMemsetAsync(ctl, 0, sizeof(uint32_t) * kJumpCtl, st));
   const unsigned nb = (m + 255) / 256;
-  // every net is walked for kWalkMin S agents; the rest of each longer
+  // every net is walked for kWalkMin round trips; the rest of each longer
   // numeral is ranked on a list of its net's agents only
-  k_nat_walk<<<nb, 256, 0, st>>>(ctx->dev, droot, m, na, nv, s_label, z_label, kWalkMin, dval, ctl);
+  k_nat_walk<<<(m + 7) / 8, 256, 0, st>>>(ctx->dev, droot, m, na, nv, s_label, z_label, kWalkMin, dval, ctl);
   CK(cudaGetLastError());
   if (na == 0) return INET_OK;
+  if (wait) {
+    uint32_t pending = 0;
+    ctx->d2h_bytes += sizeof pending;
+    CK(cudaMemcpyAsync(&pending, ctl, sizeof pending, cudaMemcpyDeviceToHost, st));
+    CK(cudaStreamSynchronize(st));
+    if (!pending) return INET_OK;
+  }
   const unsigned grid = (unsigned)std::min<uint64_t>((na + 255) / 256, 8ull * (uint64_t)std::max(ctx->num_sms, 1));
   k_nat_mark<<<nb, 256, 0, st>>>(ctx->dev, dval, m, na, mark);
   k_nat_list<<<grid, 256, 0, st>>>(ctx->dev, na, nv, s_label, z_label, mark, ctl, lst, cnt, b0);
@@ -1803,7 +1813,8 @@ inet_status inet_readback_nats(inet_ctx* ctx, const int32_t* net_ids, int32_t n,
     uint32_t* droot = at<uint32_t>(ctx, ctx->lay.rb_root);
     unsigned long long* dval = at<unsigned long long>(ctx, ctx->lay.rb_val);
     CK(h2d(ctx, droot, roots.data() + off, sizeof(uint32_t) * (size_t)m));
-    if ((s = read_nats_device(ctx, ctx->stream, droot, (uint32_t)m, si->second, zi->second, dval))) return s;
+    if ((s = read_nats_device(ctx, ctx->stream, droot, (uint32_t)m, si->second, zi->second, dval, true)))
+      return s;
     CK(d2h(ctx, values_out + off, dval, sizeof(unsigned long long) * (size_t)m));
   }
   CK(cudaStreamSynchronize(ctx->stream));
@@ -1848,7 +1859,8 @@ inet_status inet_readback_nats_begin(inet_ctx* ctx, const int32_t* net_ids, int3
     CK(cudaStreamWaitEvent(ctx->rb_stream, ctx->rb_after, 0));
     CK(cudaMemcpyAsync(droot, ctx->rb_host_roots, sizeof(uint32_t) * (size_t)n, cudaMemcpyHostToDevice,
                        ctx->rb_stream));
-    if ((s = read_nats_device(ctx, ctx->rb_stream, droot, (uint32_t)n, si->second, zi->second, dval))) return s;
+    if ((s = read_nats_device(ctx, ctx->rb_stream, droot, (uint32_t)n, si->second, zi->second, dval, false)))
+      return s;
     CK(cudaMemcpyAsync(ctx->rb_host_vals, dval, sizeof(unsigned long long) * (size_t)n, cudaMemcpyDeviceToHost,
                        ctx->rb_stream));
     CK(cudaEventRecord(ctx->rb_ready, ctx->rb_stream));
