@@ -7,6 +7,7 @@ raises at import time instead of falling back to anything else.
 """
 from __future__ import annotations
 
+import array
 import ctypes as C
 import itertools
 import os
@@ -217,15 +218,21 @@ def inet_rule_info(ctx, rule: int) -> dict:
             "n_new": d.n_new, "new_ports": d.new_ports, "n_fresh": d.n_fresh, "n_link": d.n_link}
 
 
+def _offsets(enc: list[bytes]):
+    """The n + 1 offsets of n concatenated texts, as a C array."""
+    a = array.array("Q", itertools.accumulate(map(len, enc), initial=0))
+    return (C.c_uint64 * len(a)).from_buffer(a)
+
+
 def inet_load_nets(ctx, texts) -> list[int]:
     """Loads many nets in one call (parsed on several host threads)."""
     enc = [t.encode() for t in texts]
     n = len(enc)
-    offs = (C.c_uint64 * (n + 1))(0, *itertools.accumulate(map(len, enc)))
+    offs = _offsets(enc)
     ids = (C.c_int32 * max(1, n))()
     done = C.c_int32()
     _check(ctx, LIB.inet_load_nets(ctx, b"".join(enc), offs, n, ids, C.byref(done)))
-    return list(ids[:n])
+    return ids[:n]
 
 
 def inet_parse_nets(ctx, texts) -> C.c_void_p:
@@ -233,7 +240,7 @@ def inet_parse_nets(ctx, texts) -> C.c_void_p:
     batch is freed with inet_parsed_free."""
     enc = [t.encode() for t in texts]
     n = len(enc)
-    offs = (C.c_uint64 * (n + 1))(0, *itertools.accumulate(map(len, enc)))
+    offs = _offsets(enc)
     out = C.c_void_p()
     _check(None, LIB.inet_parse_nets(ctx, b"".join(enc), offs, n, C.byref(out)))
     return out
@@ -344,9 +351,10 @@ def inet_readback(ctx, net_id: int) -> str:
     rc = LIB.inet_readback(ctx, net_id, None, 0, C.byref(need))
     if rc not in (INET_OK, INET_ERR_INVALID_ARG) or need.value == 0:
         _check(ctx, rc)
-    buf = C.create_string_buffer(need.value)
-    _check(ctx, LIB.inet_readback(ctx, net_id, buf, need.value, C.byref(need)))
-    return buf.value.decode()
+    buf = bytearray(need.value)
+    at = (C.c_char * need.value).from_buffer(buf)
+    _check(ctx, LIB.inet_readback(ctx, net_id, at, need.value, C.byref(need)))
+    return str(memoryview(buf)[:need.value - 1], "utf-8")  # a .value would look for the end byte by byte
 
 
 def inet_readback_nat(ctx, net_id: int) -> tuple[int, int]:
@@ -381,12 +389,16 @@ def inet_net_finished(ctx, cap: int = READ_CHUNK) -> list[int]:
 
 def inet_readback_nats(ctx, net_ids) -> tuple[list[int | None], list[int]]:
     """(values, interactions); a value is None when the interface is not a numeral."""
-    ids = (C.c_int32 * len(net_ids))(*net_ids)
-    vals = (C.c_uint64 * max(1, len(net_ids)))()
-    ints = (C.c_uint64 * max(1, len(net_ids)))()
-    _check(ctx, LIB.inet_readback_nats(ctx, ids, len(net_ids), vals, ints))
+    n = len(net_ids)
+    ids = (C.c_int32 * n)(*net_ids)
+    vals = (C.c_uint64 * max(1, n))()
+    ints = (C.c_uint64 * max(1, n))()
+    _check(ctx, LIB.inet_readback_nats(ctx, ids, n, vals, ints))
     none = (1 << 64) - 1
-    return [None if v == none else v for v in vals[:len(net_ids)]], list(ints[:len(net_ids)])
+    got = vals[:n]
+    if none in got:
+        got = [None if v == none else v for v in got]
+    return got, ints[:n]
 
 
 def inet_readback_nats_begin(ctx, net_ids) -> None:

@@ -9,8 +9,11 @@
 #include <cstdlib>
 #include <cstring>
 #include <map>
+#include <memory>
 #include <mutex>
+#include <new>
 #include <string>
+#include <utility>
 #include <vector>
 
 #include "host_pool.h"
@@ -103,6 +106,28 @@ Layout layout_of(const inet_arena_cfg& c) {
   return L;
 }
 
+// Vectors whose resize leaves new elements unwritten, for staging arrays that
+// the host pool fills in parallel right after (clearing 17 MB first took
+// longer than filling them).
+template <class T>
+struct Unwritten : std::allocator<T> {
+  template <class U>
+  struct rebind {
+    using other = Unwritten<U>;
+  };
+  Unwritten() = default;
+  template <class U>
+  Unwritten(const Unwritten<U>&) {}
+  template <class U>
+  void construct(U* p) {
+    ::new (static_cast<void*>(p)) U;
+  }
+  template <class U, class... A>
+  void construct(U* p, A&&... a) {
+    ::new (static_cast<void*>(p)) U(std::forward<A>(a)...);
+  }
+};
+
 struct NetRec {
   bool used = false;
   bool uploaded = false;          // its records and counter are on the device
@@ -147,11 +172,11 @@ struct inet_ctx {
   // nets
   std::vector<NetRec> nets;
   // staged loads
-  std::vector<Node> st_nodes;
+  std::vector<Node, Unwritten<Node>> st_nodes;
   uint64_t st_a0 = 0;
-  std::vector<uint32_t> st_vars;
+  std::vector<uint32_t, Unwritten<uint32_t>> st_vars;
   uint64_t st_v0 = 0;
-  std::vector<uint32_t> st_vown;            // owning net of each staged name slot
+  std::vector<uint32_t, Unwritten<uint32_t>> st_vown;            // owning net of each staged name slot
   std::vector<unsigned long long> st_netctr;
   std::vector<int32_t> st_net_ids;          // ids of the staged nets, parallel to st_netctr
   std::vector<long long> st_netlive;        // their agents, parallel to st_netctr
