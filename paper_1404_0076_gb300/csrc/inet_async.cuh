@@ -365,30 +365,6 @@ __device__ __forceinline__ bool link_async(const Dev& d, WM& W, Lane& L, int lan
   }
 }
 
-// Rule template as the asynchronous kernel reads it from shared memory: one
-// 32-bit word per new agent (label and its three port codes) and one 16-bit
-// word per equation, so an agent or an equation costs one load.
-struct AsyncTpl {
-  uint32_t hdr;                 // n_new | n_fresh << 8 | n_link << 16 | rule << 24
-  uint32_t agent[kMaxNew];      // lab | src0 << 8 | src1 << 16 | src2 << 24
-  uint16_t link[kMaxLink];      // code0 | code1 << 8
-  uint32_t inside;              // rules already applied inside: how many | rule << 8 | rule << 16
-  uint32_t pad[2];
-};
-static_assert(sizeof(AsyncTpl) == 64, "packed template is 64 bytes");
-
-__device__ __forceinline__ AsyncTpl pack_template(const Template& t, uint32_t inside = 0) {
-  AsyncTpl p;
-  p.hdr = (uint32_t)t.n_new | ((uint32_t)t.n_fresh << 8) | ((uint32_t)t.n_link << 16) | ((uint32_t)t.rule << 24);
-  for (int j = 0; j < kMaxNew; j++)
-    p.agent[j] = (uint32_t)t.lab[j] | ((uint32_t)t.src[j][0] << 8) | ((uint32_t)t.src[j][1] << 16) |
-                 ((uint32_t)t.src[j][2] << 24);
-  for (int k = 0; k < kMaxLink; k++) p.link[k] = (uint16_t)(t.link[k][0] | (t.link[k][1] << 8));
-  p.inside = inside;
-  p.pad[0] = p.pad[1] = 0;
-  return p;
-}
-
 // What one lane's step leaves: new active pairs in W.out[0 .. np)[lane],
 // equations to link after the fence in W.eq[0 .. ne)[lane], how many times
 // the rule was applied, and, when fwd is set, the records of pair 0 (ra always,
@@ -1049,7 +1025,7 @@ __device__ __forceinline__ void pass_rule(const Dev& d, WM& W, Lane& L, int lane
 // The templates of the rules with their own code (which may hold reduced
 // pairs) in place of the loaded ones.
 template <class Rules, int I = 0>
-__device__ __forceinline__ void spec_templates(AsyncTpl* tmpl) {
+__device__ __forceinline__ void spec_templates(PackedTpl* tmpl) {
   if constexpr (I < Rules::kN && I < kSpecialisedMaxRules) {
     constexpr Template R = Rules::kT[I];
     constexpr uint32_t kIn = Rules::kMore[I][0] | (Rules::kMore[I][1] << 8) | (Rules::kMore[I][2] << 16);
@@ -1072,7 +1048,7 @@ __device__ constexpr uint32_t run_mask() {
 // finds each where it is: the arguments in
 // registers, the new slots on top of the lane's columns.
 template <bool kTrack, class WM>
-__device__ __forceinline__ void interpret(const Dev& d, WM& W, Lane& L, int lane, const AsyncTpl& T, uint32_t a,
+__device__ __forceinline__ void interpret(const Dev& d, WM& W, Lane& L, int lane, const PackedTpl& T, uint32_t a,
                                           uint32_t b, const int4& ra, const int4& rb, uint32_t net, Step& S) {
   const uint32_t hdr = T.hdr;
   const uint32_t n_new = hdr & 0xFFu, n_fresh = (hdr >> 8) & 0xFFu, n_link = (hdr >> 16) & 0xFFu;
@@ -1151,7 +1127,7 @@ __device__ __forceinline__ void spec_rule(const Dev& d, WM& W, Lane& L, int lane
 // W.out[0..S.np)[lane]; a pair that cannot be reduced (no rule, corrupt
 // state) is dropped.
 template <bool kTrack, class Rules, class WM>
-__device__ __forceinline__ void async_interact(const Dev& d, const AsyncTpl* tmpl, const int16_t* tab,
+__device__ __forceinline__ void async_interact(const Dev& d, const PackedTpl* tmpl, const int16_t* tab,
                                                uint32_t* hist, WM& W, Lane& L, bool valid, uint32_t a,
                                                uint32_t b, bool pre, int4 ra, int4 rb, Step& S) {
   const int lane = threadIdx.x & 31;
@@ -1305,7 +1281,7 @@ __global__ void __launch_bounds__(256, 2) k_async(Dev d) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   size_t off = 0;
   auto take = [&](size_t n) { off = (off + 15) / 16 * 16; unsigned char* p = smem_raw + off; off += n; return p; };
-  AsyncTpl* tmpl = reinterpret_cast<AsyncTpl*>(take(sizeof(AsyncTpl) * (d.n_tmpl ? d.n_tmpl : 1)));
+  PackedTpl* tmpl = reinterpret_cast<PackedTpl*>(take(sizeof(PackedTpl) * (d.n_tmpl ? d.n_tmpl : 1)));
   using WM = WarpMem<Rules::kN == 0>;
   WM* wm = reinterpret_cast<WM*>(take(sizeof(WM) * (blockDim.x / 32)));
   uint32_t* hist = reinterpret_cast<uint32_t*>(take(sizeof(uint32_t) * INET_MAX_RULES));

@@ -157,11 +157,35 @@ __device__ __forceinline__ void set_error(Ctrl* c, int32_t code, uint32_t info) 
   if (code != INET_ERR_NO_RULE) atomicCAS(reinterpret_cast<int*>(&c->fatal), 0, code);
 }
 
+// Rule template as the kernels read it from shared memory: one
+// 32-bit word per new agent (label and its three port codes) and one 16-bit
+// word per equation, so an agent or an equation costs one load.
+struct PackedTpl {
+  uint32_t hdr;                 // n_new | n_fresh << 8 | n_link << 16 | rule << 24
+  uint32_t agent[kMaxNew];      // lab | src0 << 8 | src1 << 16 | src2 << 24
+  uint16_t link[kMaxLink];      // code0 | code1 << 8
+  uint32_t inside;              // rules already applied inside: how many | rule << 8 | rule << 16
+  uint32_t pad[2];
+};
+static_assert(sizeof(PackedTpl) == 64, "packed template is 64 bytes");
+
+__device__ __forceinline__ PackedTpl pack_template(const Template& t, uint32_t inside = 0) {
+  PackedTpl p;
+  p.hdr = (uint32_t)t.n_new | ((uint32_t)t.n_fresh << 8) | ((uint32_t)t.n_link << 16) | ((uint32_t)t.rule << 24);
+  for (int j = 0; j < kMaxNew; j++)
+    p.agent[j] = (uint32_t)t.lab[j] | ((uint32_t)t.src[j][0] << 8) | ((uint32_t)t.src[j][1] << 16) |
+                 ((uint32_t)t.src[j][2] << 24);
+  for (int k = 0; k < kMaxLink; k++) p.link[k] = (uint16_t)(t.link[k][0] | (t.link[k][1] << 8));
+  p.inside = inside;
+  p.pad[0] = p.pad[1] = 0;
+  return p;
+}
+
 // ---------------------------------------------------------------------------
 // Shared memory of one block.
 
 struct Smem {
-  Template* tmpl;            // n_tmpl
+  PackedTpl* tmpl;           // n_tmpl
   unsigned long long* warp;  // scan slots and 64-bit broadcast values
   Pair* push;                // kMaxLink * blockDim: staged new pairs (wide steps)
   uint32_t* vals;            // kNumVals * blockDim: per-thread value table
@@ -197,7 +221,7 @@ enum {
 __host__ __device__ inline size_t smem_bytes(uint32_t block, uint32_t n_labels, uint32_t n_tmpl, uint32_t solo_cap) {
   size_t b = 0;
   auto take = [&](size_t n, size_t align) { b = (b + align - 1) / align * align; b += n; };
-  take(sizeof(Template) * (n_tmpl ? n_tmpl : 1), 16);
+  take(sizeof(PackedTpl) * (n_tmpl ? n_tmpl : 1), 16);
   take(sizeof(unsigned long long) * W_SLOTS, 16);
   take(sizeof(Pair) * kMaxLink * block, 16);
   take(sizeof(uint32_t) * kNumVals * block, 16);
@@ -224,7 +248,7 @@ __device__ __forceinline__ Smem carve(const Dev& d, uint32_t solo_cap) {
   };
   Smem s;
   const uint32_t B = blockDim.x;
-  s.tmpl = reinterpret_cast<Template*>(take(sizeof(Template) * (d.n_tmpl ? d.n_tmpl : 1), 16));
+  s.tmpl = reinterpret_cast<PackedTpl*>(take(sizeof(PackedTpl) * (d.n_tmpl ? d.n_tmpl : 1), 16));
   s.warp = reinterpret_cast<unsigned long long*>(take(sizeof(unsigned long long) * W_SLOTS, 16));
   s.push = reinterpret_cast<Pair*>(take(sizeof(Pair) * kMaxLink * B, 16));
   s.vals = reinterpret_cast<uint32_t*>(take(sizeof(uint32_t) * kNumVals * B, 16));
@@ -241,9 +265,7 @@ __device__ __forceinline__ Smem carve(const Dev& d, uint32_t solo_cap) {
 }
 
 __device__ void load_tables(const Dev& d, const Smem& s) {
-  const uint32_t nt = d.n_tmpl * (sizeof(Template) / 16);
-  for (uint32_t i = threadIdx.x; i < nt; i += blockDim.x)
-    reinterpret_cast<int4*>(s.tmpl)[i] = reinterpret_cast<const int4*>(d.tmpl)[i];
+  for (uint32_t i = threadIdx.x; i < d.n_tmpl; i += blockDim.x) s.tmpl[i] = pack_template(d.tmpl[i]);
   for (uint32_t i = threadIdx.x; i < d.n_labels * d.n_labels; i += blockDim.x) s.tab[i] = d.table[i];
   for (uint32_t i = threadIdx.x; i < d.n_labels; i += blockDim.x) s.arity[i] = d.arity[i];
   for (uint32_t i = threadIdx.x; i < INET_MAX_RULES; i += blockDim.x) s.hist[i] = 0;
@@ -346,6 +368,20 @@ __device__ __forceinline__ uint32_t pool_slot(const uint32_t* ring, unsigned lon
   return (uint32_t)(bump_base + (k - ring_avail));
 }
 
+// A finished name slot is cleared and staged to be freed.
+template <bool kTrack>
+__device__ __forceinline__ void free_name(const Dev& d, const Smem& s, uint32_t x) {
+  __stcg(d.var + x, kEmpty);
+  if constexpr (kTrack) __stcg(d.vown + x, kNoNet);
+  const int pos = atomicAdd(&s.misc[M_NVSTAGE], 1);
+  if (pos < kVarStage * (int)blockDim.x) {
+    s.vstage[pos] = x;
+  } else {
+    const unsigned long long tpos = atomicAdd(&d.ctrl->v_tail, 1ull);
+    __stcg(d.vfree + tpos % d.cap_vars, x);
+  }
+}
+
 // ->com on name slots (Sec. 2.2, Communication; Sec. 3.5-3.6).  Links the
 // equation t = u.  Two agents form an active pair.  Otherwise the equation
 // arrives at a name slot x (t or u a name): the first arrival stores its
@@ -381,16 +417,7 @@ __device__ __forceinline__ bool link_eq(const Dev& d, const Smem& s, uint32_t t,
     const uint32_t x = idx_of(t);
     const uint32_t old = atomicExch(d.var + x, u);
     if (old == kEmpty) return false;
-    // second arrival: the slot is finished; clear it and free it
-    __stcg(d.var + x, kEmpty);
-    if constexpr (kTrack) __stcg(d.vown + x, kNoNet);
-    const int pos = atomicAdd(&s.misc[M_NVSTAGE], 1);
-    if (pos < kVarStage * (int)blockDim.x) {
-      s.vstage[pos] = x;
-    } else {
-      const unsigned long long tpos = atomicAdd(&d.ctrl->v_tail, 1ull);
-      __stcg(d.vfree + tpos % d.cap_vars, x);
-    }
+    free_name<kTrack>(d, s, x);  // second arrival: the slot is finished
     t = old;
   }
 }
@@ -450,9 +477,9 @@ __device__ void process_chunk(const Dev& d, const Smem& s, uint32_t base, uint32
       ti = (uint32_t)e >> 1;
     }
   }
-  const Template& T = s.tmpl[ti];
-  const uint32_t n_new = valid ? T.n_new : 0u;
-  const uint32_t n_fresh = valid ? T.n_fresh : 0u;
+  const PackedTpl& T = s.tmpl[ti];
+  const uint32_t hdr = valid ? T.hdr : 0u, rule = hdr >> 24;
+  const uint32_t n_new = hdr & 0xFFu, n_fresh = (hdr >> 8) & 0xFFu;
   // a3: allocation.  Consumed slots a and b are reused in place for the
   // first two new agents; the rest comes from the block's stacks, then the
   // global pools.
@@ -519,35 +546,24 @@ __device__ void process_chunk(const Dev& d, const Smem& s, uint32_t base, uint32
     vals[(kValExt + 4) * B] = (uint32_t)rb.z;
     vals[(kValExt + 5) * B] = (uint32_t)rb.w;
     bool in_range = true;
-#pragma unroll
-    for (int j = 0; j < kMaxNew; j++) {
-      if ((uint32_t)j < n_new) {
-        uint32_t sl;
-        if (j == 0) {
-          sl = a;
-        } else if (j == 1) {
-          sl = b;
-        } else {
-          const uint32_t k = oa + (uint32_t)j - 2;
-          if (k < ta) sl = s.la[la0 + k];
-          else sl = pool_slot(d.afree, d.cap_agents, s.warp[W_ARING], (uint32_t)s.warp[W_AAVAIL],
-                              s.warp[W_ABUMP], k - ta);
-          if (sl >= d.cap_agents) in_range = false;
-        }
-        vals[(kValNew + j) * B] = mk_agent(sl);
-      }
+    if (n_new > 0) vals[(kValNew + 0) * B] = mk_agent(a);
+    if (n_new > 1) vals[(kValNew + 1) * B] = mk_agent(b);
+    for (uint32_t j = 2; j < n_new; j++) {
+      const uint32_t k = oa + j - 2;
+      const uint32_t sl = k < ta ? s.la[la0 + k]
+                                 : pool_slot(d.afree, d.cap_agents, s.warp[W_ARING], (uint32_t)s.warp[W_AAVAIL],
+                                             s.warp[W_ABUMP], k - ta);
+      if (sl >= d.cap_agents) in_range = false;
+      vals[(kValNew + j) * B] = mk_agent(sl);
     }
-#pragma unroll
-    for (int v = 0; v < kMaxFresh; v++) {
-      if ((uint32_t)v < n_fresh) {
-        const uint32_t k = ov + (uint32_t)v;
-        uint32_t x;
-        if (k < tv) x = s.lv[lv0 + k];
-        else x = pool_slot(d.vfree, d.cap_vars, s.warp[W_VRING], (uint32_t)s.warp[W_VAVAIL], s.warp[W_VBUMP], k - tv);
-        if (x >= d.cap_vars) in_range = false;
-        else if constexpr (kTrack) __stcg(d.vown + x, net);  // the owner, before the name is published
-        vals[(kValFresh + v) * B] = mk_var(x);
-      }
+    for (uint32_t v = 0; v < n_fresh; v++) {
+      const uint32_t k = ov + v;
+      const uint32_t x = k < tv ? s.lv[lv0 + k]
+                                : pool_slot(d.vfree, d.cap_vars, s.warp[W_VRING], (uint32_t)s.warp[W_VAVAIL],
+                                            s.warp[W_VBUMP], k - tv);
+      if (x >= d.cap_vars) in_range = false;
+      else if constexpr (kTrack) __stcg(d.vown + x, net);  // the owner, before the name is published
+      vals[(kValFresh + v) * B] = mk_var(x);
     }
     if (!in_range) {
       set_error(c, INET_ERR_STATE, 4);
@@ -555,20 +571,18 @@ __device__ void process_chunk(const Dev& d, const Smem& s, uint32_t base, uint32
     }
   }
   if (valid) {
-    const int32_t head_net = (int32_t)(net << 8);
-#pragma unroll
-    for (int j = 0; j < kMaxNew; j++) {
-      if ((uint32_t)j < n_new) {
-        const uint8_t c0 = T.src[j][0], c1 = T.src[j][1], c2 = T.src[j][2];
-        int4 rec;
-        rec.x = head_net | (int32_t)T.lab[j];
-        rec.y = c0 == kValNone ? 0 : (int32_t)vals[c0 * B];
-        rec.z = c1 == kValNone ? 0 : (int32_t)vals[c1 * B];
-        rec.w = c2 == kValNone ? 0 : (int32_t)vals[c2 * B];
-        st_node(d.node + idx_of(vals[(kValNew + j) * B]), rec);
-      }
+    const uint32_t head_net = net << 8;
+    auto port = [&](uint32_t code) -> int32_t { return code == kValNone ? 0 : (int32_t)vals[code * B]; };
+    for (uint32_t j = 0; j < n_new; j++) {
+      const uint32_t w = T.agent[j];
+      int4 rec;
+      rec.x = (int32_t)(head_net | (w & 0xFFu));
+      rec.y = port((w >> 8) & 0xFFu);
+      rec.z = port((w >> 16) & 0xFFu);
+      rec.w = port(w >> 24);
+      st_node(d.node + idx_of(vals[(kValNew + j) * B]), rec);
     }
-    n_link = T.n_link;
+    n_link = (hdr >> 16) & 0xFFu;
   }
   // a4 + a5: link the equations of Theta' and compact the new active pairs
   // (warp ballot + popc, one shared reservation per warp; in wide steps one
@@ -581,10 +595,37 @@ __device__ void process_chunk(const Dev& d, const Smem& s, uint32_t base, uint32
   if (d.paper && i < n)
     for (uint32_t k = 0; k < d.eq_fix_n; k++)
       if (slot0 + k < d.cap_fix) d.eq_fix[slot0 + k] = 0ull;
-  for (uint32_t k = 0; k < max_link; k++) {
-    Pair out;
-    bool has = false;
-    if (k < n_link) has = link_eq<kTrack>(d, s, vals[T.link[k][0] * B], vals[T.link[k][1] * B], &out, slot0 + k);
+  // the first exchanges of the first kBatch equations back to back, then what
+  // each found.  A step is a chain of round trips (frontier, records, slots,
+  // exchanges, the reservation of the new pairs) and block barriers, about
+  // 17 000 cycles for one chunk of 256 pairs; one round trip for the exchanges
+  // instead of three, and loops over what a rule has instead of over the most
+  // a rule may have, took it from 9.8 to 8.9 us a step (333 Mul nets, 1329
+  // steps: 13.0 -> 11.9 ms; graph loop on 2048: 84 -> 73 ms; plain: 177 -> 158).
+  constexpr uint32_t kBatch = 3;
+  uint32_t lt[kBatch], lu[kBatch], lo[kBatch];
+  if (!d.paper) {
+#pragma unroll
+    for (uint32_t k = 0; k < kBatch; k++) {
+      lo[k] = kEmpty;
+      if (k < n_link) {
+        const uint32_t lk = T.link[k];
+        uint32_t t = vals[(lk & 0xFFu) * B], u = vals[(lk >> 8) * B];
+        if (!is_var(t)) {
+          const uint32_t w = t;
+          t = u;
+          u = w;
+        }
+        if (is_var(t)) {
+          if (idx_of(t) < d.cap_vars) lo[k] = atomicExch(d.var + idx_of(t), u);
+          else set_error(d.ctrl, INET_ERR_STATE, 1);
+        }
+        lt[k] = t;
+        lu[k] = u;
+      }
+    }
+  }
+  auto push = [&](bool has, const Pair& out) {
     const unsigned m = __ballot_sync(kFull, has);
     if (m) {
       const int leader = __ffs(m) - 1;
@@ -598,6 +639,34 @@ __device__ void process_chunk(const Dev& d, const Smem& s, uint32_t base, uint32
       }
     }
     pushed += has ? 1u : 0u;
+  };
+  if (!d.paper) {
+#pragma unroll
+    for (uint32_t k = 0; k < kBatch; k++) {
+      if (k >= max_link) break;
+      Pair out;
+      bool has = false;
+      if (k < n_link) {
+        if (is_agent(lt[k]) && is_agent(lu[k])) {
+          out = Pair{idx_of(lt[k]), idx_of(lu[k])};
+          has = true;
+        } else if (lo[k] != kEmpty) {
+          // second arrival: the slot is finished; go on with old = u
+          free_name<kTrack>(d, s, idx_of(lt[k]));
+          has = link_eq<kTrack>(d, s, lo[k], lu[k], &out, 0);
+        }
+      }
+      push(has, out);
+    }
+  }
+  for (uint32_t k = d.paper ? 0u : kBatch; k < max_link; k++) {
+    Pair out;
+    bool has = false;
+    if (k < n_link) {
+      const uint32_t lk = T.link[k];
+      has = link_eq<kTrack>(d, s, vals[(lk & 0xFFu) * B], vals[(lk >> 8) * B], &out, slot0 + k);
+    }
+    push(has, out);
   }
   // a6: per-net counters (interactions, pending pairs) and the rule histogram
   const unsigned vm = __ballot_sync(kFull, valid);
@@ -617,8 +686,8 @@ __device__ void process_chunk(const Dev& d, const Smem& s, uint32_t base, uint32
       if (n_new != 2) atomicAdd(reinterpret_cast<unsigned long long*>(d.netlive + net),
                                 (unsigned long long)((long long)n_new - 2));
     }
-    const unsigned rp = __match_any_sync(vm, (unsigned)T.rule);
-    if (lane == __ffs(rp) - 1) atomicAdd(&s.hist[T.rule], (uint32_t)__popc(rp));
+    const unsigned rp = __match_any_sync(vm, rule);
+    if (lane == __ffs(rp) - 1) atomicAdd(&s.hist[rule], (uint32_t)__popc(rp));
   }
   __syncthreads();
   if (tid == 0) {
@@ -745,9 +814,13 @@ __device__ void finalize_step(const Dev& d) {
 }
 
 // One step of the loop; the last block to finish runs finalize_step().
-// Used by the plain host loop and by the CUDA-graph loop.
+// Used by the plain host loop and by the CUDA-graph loop.  At most 512
+// threads, one block of them per SM: 128 registers a thread, which the
+// exchanges in flight need (with 64, chosen for two such blocks, they spill:
+// 333 Mul nets in the persistent kernel 13.6 ms instead of 11.9, 2048 in the
+// graph loop 90 instead of 73).
 template <bool kTrack>
-__global__ void __launch_bounds__(512) k_step(Dev d) {
+__global__ void __launch_bounds__(512, 1) k_step(Dev d) {
   Smem s = carve(d, 0);
   load_tables(d, s);
   Ctrl* c = d.ctrl;
@@ -941,7 +1014,7 @@ __device__ void solo_phase(const Dev& d, const Smem& s, uint32_t n, uint32_t gcu
 }
 
 template <bool kTrack>
-__global__ void __launch_bounds__(512) k_persistent(Dev d) {
+__global__ void __launch_bounds__(512, 1) k_persistent(Dev d) {
   Smem s = carve(d, d.solo_max);
   load_tables(d, s);
   Ctrl* c = d.ctrl;
