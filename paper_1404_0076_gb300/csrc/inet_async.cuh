@@ -1329,10 +1329,11 @@ __global__ void __launch_bounds__(256, 2) k_async(Dev d) {
     t_start = ld_volatile64(&c->slice_t0);
   }
   for (uint32_t it = 0;; it++) {
-    // stop / slice checks every 16 iterations (on flags loaded during the
-    // iteration before), and when a napping warp's clock says the time
+    // stop / slice checks every 4 iterations (on flags loaded during the
+    // iteration before; an iteration may hold a run, and with 16 a slice of
+    // 250 us took 2.2 ms on Fibonacci(22..25) x 64, now 0.56), and when a napping warp's clock says the time
     // slice is over
-    if ((it & 15) == 15 || check_now) {
+    if ((it & 3) == 3 || check_now) {
       if (check_now) {
         if (lane == 1) flag = ld_volatile(&c->astop);
         if (lane == 2) flag = ld_volatile((const uint32_t*)&c->fatal);
@@ -1415,7 +1416,7 @@ __global__ void __launch_bounds__(256, 2) k_async(Dev d) {
       continue;
     }
     nap = 0;
-    if ((it & 15) == 14) {
+    if ((it & 3) == 2) {
       if (lane == 1) flag = ld_volatile(&c->astop);
       if (lane == 2) flag = ld_volatile((const uint32_t*)&c->fatal);
     }
