@@ -744,15 +744,20 @@ inet_status read_text_device(inet_ctx* ctx, int32_t id, std::string& out, bool* 
                                                                 ctx->dev.arity, parent, ctl);
   k_txt_init<<<grid_for(std::max(n_c, nroots)), 256, 0, st>>>(ctx->dev, n_c, na, nv, slot, cid, droots, nroots,
                                                               ctx->dev.arity, lablen, parent, b0, b1, ctl);
-  // the head of the list (root 0's first element) into ctl[2]
-  k_txt_head<<<1, 1, 0, st>>>(ctx->dev, n_c, na, nv, cid, droots, ctl);
   uint32_t rounds = 1;
   while (rounds < 64 && (1ull << rounds) < (uint64_t)n_el) rounds++;
-  for (uint32_t r = 0; r < rounds && 8 + r < (uint32_t)kTxtCtl; r++) {
-    k_txt_round<<<gel, 256, 0, st>>>(n_el, r, ctl, b0, b1);
-    k_txt_check_head<<<1, 1, 0, st>>>(n_el, r, ctl, b0, b1);
+  TxtElem* dhead = reinterpret_cast<TxtElem*>(ctl + kTxtCtl);
+  if (n_el <= kTxtShort) {
+    k_txt_rank_short<<<1, 1024, 0, st>>>(ctx->dev, n_c, na, nv, cid, droots, n_el, rounds, ctl, b0, b1, dhead);
+  } else {
+    // the head of the list (root 0's first element) into ctl[2]
+    k_txt_head<<<1, 1, 0, st>>>(ctx->dev, n_c, na, nv, cid, droots, ctl);
+    for (uint32_t r = 0; r < rounds && 8 + r < (uint32_t)kTxtCtl; r++) {
+      k_txt_round<<<gel, 256, 0, st>>>(n_el, r, ctl, b0, b1);
+      k_txt_check_head<<<1, 1, 0, st>>>(n_el, r, ctl, b0, b1);
+    }
+    k_txt_copy_head<<<1, 1, 0, st>>>(ctl, b0, b1, dhead);
   }
-  k_txt_copy_head<<<1, 1, 0, st>>>(ctl, b0, b1, reinterpret_cast<TxtElem*>(ctl + kTxtCtl));
   CK(cudaGetLastError());
   static thread_local uint32_t hctl[kTxtCtl + 2 * sizeof(TxtElem) / 4];
   CK(d2h(ctx, hctl, ctl, sizeof(uint32_t) * kTxtCtl + sizeof(TxtElem)));
