@@ -516,7 +516,9 @@ def main():
                              "frac": depth * per_level * 1e-9 / step_s,
                              "lone_chain_ns_per_interaction": lone,
                              "frac_of_lone_chain": depth * lone * 1e-9 / step_s if lone else None,
-                             "how": "depth = steps of the maximally parallel loop (persistent form) on the same batch; "
+                             "how": "depth = steps of the maximally parallel loop (persistent form) on the same batch "
+                                    "(the asynchronous kernel's runs pass many levels with one fence and exchange, "
+                                    "so frac can exceed 1); "
                                     "ns_per_level = timed device time per step / depth; bound = depth x the hardware "
                                     "floor of one level (inet_bench_chase: one thread storing a record, fencing, "
                                     "exchanging a name slot and loading the record the exchange names, 2^16 dependent "
