@@ -307,7 +307,7 @@ class Server:
         wake = threading.Event()
         stop = threading.Event()
         err = []
-        ahead = [0]                      # requests parsed and not yet admitted
+        ahead = [0]                      # requests parsed, or being parsed, and not yet admitted
 
         def parser():
             try:
@@ -316,6 +316,7 @@ class Server:
                         room = ahead[0] < 65536
                         batch, nbytes = [], 0
                         while room and to_parse and len(batch) < 2048 and nbytes < (8 << 20):
+                            ahead[0] += 1   # before it leaves the queue: serve() ends when both are empty
                             rid, r = to_parse.popleft()
                             batch.append((rid, r))
                             nbytes += r.size
@@ -327,7 +328,6 @@ class Server:
                     p = self.ev.parse([t for _, t, _, _ in rows])
                     with lock:
                         parsed.append({"reqs": rows, "parsed": p, "next": 0})
-                        ahead[0] += len(rows)
             except BaseException as e:  # surfaced on the serving thread
                 err.append(e)
 
