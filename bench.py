@@ -487,7 +487,8 @@ def main():
                        "exch_per_interaction_max": exch_per_int,
                        "interactions_per_s_bound": ex_hbm / max(1e-9, exch_per_int),
                        "frac": value / (ex_hbm / max(1e-9, exch_per_int)),
-                       "how": "inet_bench_exch: random 32-bit atomicExch returning the old value, 16 MiB and 4 GiB arrays"}
+                       "how": "inet_bench_exch: random 32-bit atomicExch returning the old value, 16 MiB and 4 GiB "
+                              "arrays; interactions inside a run along a list make no exchange"}
     prepared()
     stp_depth = ev.reduce([], mode="persistent")
     depth = stp_depth["steps"]
