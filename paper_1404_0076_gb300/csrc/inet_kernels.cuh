@@ -619,6 +619,8 @@ __device__ void process_chunk(const Dev& d, const Smem& s, uint32_t base, uint32
         if (is_var(t)) {
           if (idx_of(t) < d.cap_vars) lo[k] = atomicExch(d.var + idx_of(t), u);
           else set_error(d.ctrl, INET_ERR_STATE, 1);
+        } else if (!is_agent(t) || !is_agent(u)) {
+          set_error(d.ctrl, INET_ERR_STATE, 1);  // a word that is neither (link_eq's check)
         }
         lt[k] = t;
         lu[k] = u;
