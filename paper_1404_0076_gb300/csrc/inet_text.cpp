@@ -562,7 +562,7 @@ struct CharClass {
   uint8_t of[256];
   CharClass() {
     memset(of, 0, sizeof of);
-    for (unsigned char c : {' ', '\t', '\n', '\v', '\f', '\r'}) of[c] = kBlank;
+    for (unsigned char c : {' ', '\t', '\n', '\v', '\f', '\r', '#'}) of[c] = kBlank;  // '#' begins a comment
     for (int c = 'A'; c <= 'Z'; c++) of[c] = kUpper | kWord;
     for (int c = 'a'; c <= 'z'; c++) of[c] = kLower | kWord;
     for (int c = '0'; c <= '9'; c++) of[c] = kWord;
@@ -572,10 +572,11 @@ struct CharClass {
 const CharClass kChars;
 
 // The same pass over a well-formed net, with nothing on the way but what such
-// a net needs (no messages, no offsets, no comments).  False, with `out`
-// unspecified, for any text that is not plainly one: NetReader reads it again
-// and says what is wrong.  The work space is kept by the thread, so that a net
-// costs one allocation of its size.  What bounds it: the characters, one core
+// a net needs (no messages, no offsets).  False, with `out` unspecified, for a
+// text with an error: NetReader reads it again and says what is wrong.  The
+// work space is kept by the thread, so that a net costs one allocation of its
+// size.  Names are looked up by a scan while they are few and through a hash
+// table from kScan on.  What bounds it: the characters, one core
 // each (4096 sums, 3.3 MB of text, on 16 cores: loading 5.5 -> 3.1 ms, of which
 // a third is the caller's list of texts; 20 000 nested S on one: 0.73 -> 0.25).
 struct PlainReader {
@@ -591,6 +592,7 @@ struct PlainReader {
     std::vector<Frame> frames;
     std::vector<std::pair<const char*, uint32_t>> names;  // text and length, in order of first occurrence
     std::vector<uint8_t> count;
+    std::vector<uint32_t> table;                           // open addressing, name + 1 or 0: no entry; a power of two
     int16_t one[256];                                      // label of a one-letter symbol, -1: none
   };
   static Work& work() {
@@ -604,13 +606,57 @@ struct PlainReader {
 
   static uint8_t cls(char c) { return kChars.of[(unsigned char)c]; }
   char peek() {
-    while (p < end && (cls(*p) & kBlank)) p++;
+    while (p < end && (cls(*p) & kBlank)) {
+      if (*p++ == '#')
+        while (p < end && *p != '\n') p++;
+    }
     return p < end ? *p : '\0';
   }
   bool take(char c) {
     if (peek() != c) return false;
     p++;
     return true;
+  }
+
+  // The number of the name at b, a new one if it has not occurred.
+  static constexpr uint32_t kScan = 16;
+  bool same(uint32_t v, const char* b, uint32_t len) const {
+    return W.names[v].second == len && memcmp(W.names[v].first, b, len) == 0;
+  }
+  size_t place(const char* b, uint32_t len) const {
+    uint64_t h = 0xcbf29ce484222325ull;  // FNV-1a
+    for (uint32_t i = 0; i < len; i++) h = (h ^ (unsigned char)b[i]) * 0x100000001b3ull;
+    return (size_t)(h ^ (h >> 32)) & (W.table.size() - 1);
+  }
+  // kScan names or more: the entry of the table, made if there is none.
+  __attribute__((noinline)) uint32_t hashed(const char* b, uint32_t len) {
+    const uint32_t n = (uint32_t)W.names.size();
+    if (n == kScan || 2 * (size_t)n >= W.table.size()) {
+      W.table.assign(n == kScan ? 8 * kScan : 2 * W.table.size(), 0u);
+      for (uint32_t v = 0; v < n; v++) {
+        size_t a = place(W.names[v].first, W.names[v].second);
+        while (W.table[a]) a = (a + 1) & (W.table.size() - 1);
+        W.table[a] = v + 1;
+      }
+    }
+    size_t at = place(b, len);
+    for (; W.table[at]; at = (at + 1) & (W.table.size() - 1))
+      if (same(W.table[at] - 1, b, len)) return W.table[at] - 1;
+    W.table[at] = n + 1;
+    return n;
+  }
+  uint32_t name(const char* b, uint32_t len) {
+    const uint32_t n = (uint32_t)W.names.size();
+    uint32_t v = 0;
+    if (n <= kScan)
+      while (v < n && !same(v, b, len)) v++;
+    if (n >= kScan && (n > kScan || v == n)) v = hashed(b, len);
+    if (v == n) {
+      W.names.emplace_back(b, len);
+      W.count.push_back(0);
+      out.vars.push_back(kEmpty);
+    }
+    return v;
   }
 
   bool term(uint32_t* w_out) {
@@ -626,15 +672,7 @@ struct PlainReader {
       int32_t arity = 0;
       bool opened = false;
       if (k & kLower) {
-        uint32_t v = 0;
-        const uint32_t n = (uint32_t)W.names.size();
-        while (v < n && !(W.names[v].second == len && memcmp(W.names[v].first, b, len) == 0)) v++;
-        if (v == n) {
-          if (n >= 32) return false;  // many names: a hash table serves better
-          W.names.emplace_back(b, len);
-          W.count.push_back(0);
-          out.vars.push_back(kEmpty);
-        }
+        const uint32_t v = name(b, len);
         if (++W.count[v] > 2) return false;
         w = mk_var(var_base + v);
       } else {
