@@ -191,9 +191,16 @@ __device__ __forceinline__ uint32_t take_name(const Dev& d, const WM& W, Lane& L
 }
 
 // One pop of the global pools for the warp's stacks (ac agents, vc names
-// now): up to Ka and Kv and a few more, or what half of the room above the
-// bump pointer divided among the grid's warps allows, but at least up to
-// Ma and Mv, which one step needs.  Returns false when the arena is full
+// now): up to Ka and Kv and a few more, but no more than a warp's share of
+// half of what is left, in the ring of recycled slots and above the bump
+// pointer together, so that no warp starves the others, and from the bump
+// pointer no more than a share of its own room; but at least what one step
+// needs (Ma, Mv), and no more agents than that once a share is below 32, when
+// what warps keep for later is what the nets lack (256 Mul nets then reduce
+// over and over in 1.06 times their peak, else in 1.12).  With a share of the
+// bump pointer's room alone, every pop of a context that runs on recycled slots
+// was a bare step's need: 2048 Mul nets loaded, reduced and freed over and over
+// in 1.1 times their peak 9.0 ms, now 5.5.  Returns false when the arena is full
 // (fatal: the loop stops).  Warp-collective.
 template <class WM>
 __device__ __noinline__ bool fill_stacks(const Dev& d, WM& W, uint32_t ac, uint32_t vc, uint32_t Ka, uint32_t Kv,
@@ -213,22 +220,30 @@ __device__ __noinline__ bool fill_stacks(const Dev& d, WM& W, uint32_t ac, uint3
   unsigned long long rb = 0, bb = 0;
   if (lane < 2 && want > have) {
     const unsigned long long room = bump < cap ? cap - bump : 0ull;
-    const unsigned long long warps = (unsigned long long)gridDim.x * (blockDim.x / 32);
+    const unsigned long long ring = cnt < pub ? pub - cnt : 0ull;  // a ring seen empty is left alone
+    const unsigned long long shares = 2ull * gridDim.x * (blockDim.x / 32);
+    const uint32_t need = least > have ? least - have : 0u;
     k = want - have + (lane == 0 ? kFetchA : kFetchV);
-    if (room < 2 * k * warps) k = max((uint32_t)(room / (2 * warps)), least > have ? least - have : 0u);
+    if (ring + room < k * shares) {
+      const uint32_t share = (uint32_t)((ring + room) / shares);
+      k = lane == 0 && share < 32 ? need : max(share, need);
+    }
     k = min(k, size - have);
-    if (k && cnt < pub) {  // a ring seen empty is left alone
+    if (k && ring) {
       const unsigned long long h = atomicAdd(lane == 0 ? &c->a_head : &c->v_head, (unsigned long long)k);
       av = h < pub ? (uint32_t)min((unsigned long long)k, pub - h) : 0u;
       rb = h % cap;
     }
-    if (av < k) {
-      bb = atomicAdd(lane == 0 ? &c->a_bump : &c->v_bump, (unsigned long long)(k - av));
-      if (bb + (k - av) > cap) {
+    uint32_t u = k - av;
+    if (room < u * shares) u = max((uint32_t)(room / shares), need > av ? need - av : 0u);
+    if (u) {
+      bb = atomicAdd(lane == 0 ? &c->a_bump : &c->v_bump, (unsigned long long)u);
+      if (bb + u > cap) {
         ok = 0;
         set_error(c, INET_ERR_ARENA_FULL, 0);
       }
     }
+    k = av + u;
   }
   if (!__all_sync(kFull, ok)) return false;
   // on top of the stacks, the lowest slot last, so that slots from the bump
