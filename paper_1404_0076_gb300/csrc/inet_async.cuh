@@ -52,14 +52,9 @@
 
 namespace inet {
 
-// A column of 16 agent slots lets a run of Dup go on for 16 copies and lays
-// them out side by side; 4 freed slots kept per lane (2048 Mul nets: 4.4 ms
-// with 2, 3.9 with 4, 4.3 with 8, when these were measured against each other).
-constexpr int kARes = 16;      // free agent slots a lane keeps for itself
+// 4 freed slots kept per lane: 2048 Mul nets took 12 % longer with 2, 10 % with 8.
 constexpr int kVRes = 8;       // free name slots a lane keeps for itself
 constexpr int kKeep = 4;       // slots of each kind a lane keeps of those it frees; the rest is the warp's
-constexpr int kAStack = 576;   // per-warp stack of free agent slots
-constexpr int kVStack = 288;   // per-warp stack of free name slots
 // Most interactions of one run: of a warp's only lane, of one lane among
 // several, and where most of the warp's lanes reduce rules that do not run
 // (they wait for the run).  Lone: a chain of 20 000 Add 3.4 ms with 64, 2.3
@@ -70,8 +65,6 @@ constexpr int kVStack = 288;   // per-warp stack of free name slots
 constexpr uint32_t kRunLone = 512, kRunMany = 64, kRunMixed = 16;
 constexpr unsigned long long kNoTicket = ~0ull;
 constexpr uint32_t kFetchA = 32, kFetchV = 16;  // slots fetched beyond the need when a warp's stack runs dry
-static_assert(kARes >= kMaxNew - 2 && kVRes >= kMaxFresh, "a lane's slots serve any one interaction");
-static_assert(kAStack >= 32 * kARes + (int)kFetchA && kVStack >= 32 * kVRes + (int)kFetchV, "a warp's stacks serve any one step");
 
 // Shared memory of one warp.  kTable: with the value table of the general
 // kernel, which interprets every rule.
@@ -86,6 +79,12 @@ struct ValueTable<true> {
 };
 template <bool kTable>
 struct alignas(16) WarpMem : ValueTable<kTable> {
+  // Agent slots of a lane, agents and names of the warp's stack.  A column of 16
+  // lets a run of Dup go on for 16 copies and lays them out side by side.  The
+  // general kernel has no runs: what one step of the warp can need.
+  static constexpr int kARes = kTable ? 8 : 16, kAStack = kTable ? 192 : 576, kVStack = kTable ? 256 : 288;
+  static_assert(kARes >= kMaxNew - 2 && kVRes >= kMaxFresh, "a lane's slots serve any one interaction");
+  static_assert(kAStack >= 32 * (kTable ? kMaxNew - 2 : kARes) && kVStack >= 32 * kVRes, "a warp's stacks serve any one step");
   uint32_t ares[kARes][32];      // lane-private free slots, a column per lane
   uint32_t vres[kVRes][32];
   Pair out[kMaxLink][32];        // new active pairs of one step
@@ -98,15 +97,21 @@ struct alignas(16) WarpMem : ValueTable<kTable> {
   int an, vn, pad[2];            // entries of the warp's stacks (above the size: pushes that went to the ring)
 };
 
-__host__ __device__ inline size_t async_smem_bytes(uint32_t block, uint32_t n_labels, uint32_t n_tmpl, bool table) {
+__host__ __device__ constexpr size_t async_smem_bytes(uint32_t block, uint32_t n_labels, uint32_t n_tmpl, bool table) {
   size_t b = 0;
   auto take = [&](size_t n, size_t align) { b = (b + align - 1) / align * align; b += n; };
-  take(sizeof(Template) * (n_tmpl ? n_tmpl : 1), 16);
+  take(sizeof(PackedTpl) * (n_tmpl ? n_tmpl : 1), 16);
   take((table ? sizeof(WarpMem<true>) : sizeof(WarpMem<false>)) * (block / 32), 16);
   take(sizeof(uint32_t) * INET_MAX_RULES, 16);
   take(sizeof(int16_t) * n_labels * n_labels, 16);
   return b + 16;
 }
+// Two blocks share an SM whatever the rule set: the general kernel's batch of
+// 2048 Mul nets takes 12.9 ms under 64 rules and 57 symbols, as under the 18
+// alone, where one block an SM took 16.8 (and 13.8 two that leave L1 only 28 of
+// the 256 KB, hence 97 KB).  Each block takes 1 KB besides its own.
+static_assert(async_smem_bytes(256, kMaxLabels, INET_MAX_RULES, true) <= 97 * 1024 &&
+              async_smem_bytes(256, kMaxLabels, INET_MAX_RULES, false) <= 113 * 1024, "two blocks per SM");
 
 __device__ __forceinline__ unsigned long long ld_acquire64(const unsigned long long* p) {
   unsigned long long v;
@@ -142,7 +147,7 @@ struct Lane {
 template <class WM>
 __device__ __noinline__ void spill_agent(const Dev& d, WM& W, uint32_t slot) {
   const int pos = atomicAdd(&W.an, 1);
-  if (pos < kAStack) {
+  if (pos < WM::kAStack) {
     W.astk[pos] = slot;
   } else {
     const unsigned long long tp = atomicAdd(&d.ctrl->a_tail, 1ull);
@@ -152,7 +157,7 @@ __device__ __noinline__ void spill_agent(const Dev& d, WM& W, uint32_t slot) {
 template <class WM>
 __device__ __noinline__ void spill_name(const Dev& d, WM& W, uint32_t x) {
   const int pos = atomicAdd(&W.vn, 1);
-  if (pos < kVStack) {
+  if (pos < WM::kVStack) {
     W.vstk[pos] = x;
   } else {
     const unsigned long long tp = atomicAdd(&d.ctrl->v_tail, 1ull);
@@ -215,7 +220,7 @@ __device__ __noinline__ bool fill_stacks(const Dev& d, WM& W, uint32_t ac, uint3
   const unsigned long long pub = __shfl_down_sync(kFull, cnt, 2), bump = __shfl_down_sync(kFull, cnt, 4);
   const unsigned long long cap = lane == 0 ? d.cap_agents : d.cap_vars;
   const uint32_t have = lane == 0 ? ac : vc, want = lane == 0 ? Ka : Kv, least = lane == 0 ? Ma : Mv;
-  const uint32_t size = lane == 0 ? (uint32_t)kAStack : (uint32_t)kVStack;
+  const uint32_t size = lane == 0 ? (uint32_t)WM::kAStack : (uint32_t)WM::kVStack;
   uint32_t ok = 1, av = 0, k = 0;
   unsigned long long rb = 0, bb = 0;
   if (lane < 2 && want > have) {
@@ -276,11 +281,11 @@ template <class WM>
 __device__ __forceinline__ bool refill(const Dev& d, WM& W, Lane& L, bool runs, uint32_t need_a,
                                        uint32_t need_v, int lane) {
   __syncwarp();
-  uint32_t ac = (uint32_t)min(W.an, kAStack), vc = (uint32_t)min(W.vn, kVStack);
+  uint32_t ac = (uint32_t)min(W.an, WM::kAStack), vc = (uint32_t)min(W.vn, WM::kVStack);
   // what the step needs, or more: a whole column for a run that allocates
   const uint32_t least_a = (uint32_t)L.na < need_a ? need_a - (uint32_t)L.na : 0u;
   const uint32_t least_v = (uint32_t)L.nv < need_v ? need_v - (uint32_t)L.nv : 0u;
-  uint32_t wa = least_a ? (uint32_t)(runs ? kARes : max((int)need_a, 4)) - (uint32_t)L.na : 0u;
+  uint32_t wa = least_a ? (uint32_t)(runs ? WM::kARes : max((int)need_a, 4)) - (uint32_t)L.na : 0u;
   uint32_t wv = least_v ? (uint32_t)max((int)need_v, 4) - (uint32_t)L.nv : 0u;
   uint32_t inc, packed, Ka, Kv;
   // offsets of this lane among the warp's wants
@@ -312,20 +317,20 @@ __device__ __forceinline__ bool refill(const Dev& d, WM& W, Lane& L, bool runs, 
       const uint32_t at_a = ac + ((g - own) & 0xFFFFu), at_v = vc + ((g - own) >> 16);
       uint32_t da = 0, dv = 0;
 #pragma unroll 1
-      for (; da < ga && at_a + da < (uint32_t)kAStack; da++) W.astk[at_a + da] = W.ares[--L.na][lane];
+      for (; da < ga && at_a + da < (uint32_t)WM::kAStack; da++) W.astk[at_a + da] = W.ares[--L.na][lane];
 #pragma unroll 1
-      for (; dv < gv && at_v + dv < (uint32_t)kVStack; dv++) W.vstk[at_v + dv] = W.vres[--L.nv][lane];
+      for (; dv < gv && at_v + dv < (uint32_t)WM::kVStack; dv++) W.vstk[at_v + dv] = W.vres[--L.nv][lane];
       const uint32_t tot = __shfl_sync(kFull, g, 31);
-      ac = min(ac + (tot & 0xFFFFu), (uint32_t)kAStack);
-      vc = min(vc + (tot >> 16), (uint32_t)kVStack);
+      ac = min(ac + (tot & 0xFFFFu), (uint32_t)WM::kAStack);
+      vc = min(vc + (tot >> 16), (uint32_t)WM::kVStack);
       __syncwarp();
     }
   }
   if (Ka > ac || Kv > vc) {
     const uint32_t Ma = __reduce_add_sync(kFull, least_a), Mv = __reduce_add_sync(kFull, least_v);
     if (!fill_stacks(d, W, ac, vc, Ka, Kv, Ma, Mv)) return false;
-    ac = (uint32_t)min(W.an, kAStack);
-    vc = (uint32_t)min(W.vn, kVStack);
+    ac = (uint32_t)min(W.an, WM::kAStack);
+    vc = (uint32_t)min(W.vn, WM::kVStack);
     if (Ka > ac || Kv > vc) {
       wa = least_a;
       wv = least_v;
@@ -1637,7 +1642,7 @@ __global__ void __launch_bounds__(256, 2) k_async(Dev d) {
   // may come from the bump pointer with stale contents)
   __syncwarp();
   {
-    const uint32_t ac = (uint32_t)min(W.an, kAStack), vc = (uint32_t)min(W.vn, kVStack);
+    const uint32_t ac = (uint32_t)min(W.an, WM::kAStack), vc = (uint32_t)min(W.vn, WM::kVStack);
     uint32_t inc = (uint32_t)L.na | ((uint32_t)L.nv << 16);
     const uint32_t own = inc;
 #pragma unroll
