@@ -33,3 +33,23 @@ def test_general_kernel_keeps_its_blocks_with_the_largest_rule_sets():
             got.append(device_ms(ev, nets, 5))
     assert got[0][1] == got[1][1]
     assert got[1][0] < 1.15 * got[0][0], got
+
+
+@pytest.mark.gpu
+def test_a_list_taken_one_agent_at_a_time_is_not_made_in_runs():
+    # the L-System's Dup copies numerals that only SymA and SymB take, one S at
+    # a time; with a rule that walks such lists Dup is reduced in runs, which
+    # hold the copies back (measured: 1.6 times as long)
+    import torch
+    assert torch.cuda.is_available(), "GPU tests need a GPU"
+    from paper_1404_0076_gb300 import Evaluator
+    walker = "Walk(r) = Z -> r = Z;\nWalk(r) = S(x) -> Walk(w) = x, r = S(w);\n"
+    got = []
+    for rules in (W.LSYS_RULES, W.LSYS_RULES + walker):
+        with Evaluator(device=0, jit=True, max_agents=1 << 22, max_vars=1 << 22, max_pairs=1 << 20, max_nets=64) as ev:
+            ev.load_rules(rules)
+            ev.build_jit()
+            got.append(device_ms(ev, [W.lsys_net(16)], 12))
+            assert ev.jit_info()["state"] == 1
+    assert got[0][1] == got[1][1]
+    assert got[0][0] < 0.85 * got[1][0], got
