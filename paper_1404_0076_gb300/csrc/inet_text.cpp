@@ -9,6 +9,8 @@
 #include <cstdlib>
 #include <cctype>
 #include <cstring>
+#include <memory>
+#include <mutex>
 #include <string_view>
 #include <unordered_map>
 
@@ -575,7 +577,8 @@ const CharClass kChars;
 // a net needs (no messages, no offsets).  False, with `out` unspecified, for a
 // text with an error: NetReader reads it again and says what is wrong.  The
 // work space is kept by the thread, so that a net costs one allocation of its
-// size.  Names are looked up by a scan while they are few and through a hash
+// size; what a large net needs is kept once for the process (kShared), and not
+// at all beyond that.  Names are looked up by a scan while they are few and through a hash
 // table from kScan on.  What bounds it: the characters, one core
 // each (4096 sums, 3.3 MB of text, on 16 cores: loading 5.5 -> 3.1 ms, of which
 // a third is the caller's list of texts; 20 000 nested S on one: 0.73 -> 0.25).
@@ -588,21 +591,58 @@ struct PlainReader {
     int32_t port, arity;
   };
   struct Work {
-    std::vector<Node> nodes;
+    std::unique_ptr<Node[], void (*)(void*)> nodes{nullptr, free};
+    size_t cap = 0;                                        // of nodes
     std::vector<Frame> frames;
     std::vector<std::pair<const char*, uint32_t>> names;  // text and length, in order of first occurrence
     std::vector<uint8_t> count;
     std::vector<uint32_t> table;                           // open addressing, name + 1 or 0: no entry; a power of two
+    // Room for more nodes, which grow as they are read.
+    bool grow() {
+      const size_t n = cap ? 2 * cap : 4096;
+      void* p = realloc(nodes.get(), n * sizeof(Node));
+      if (!p) return false;
+      nodes.release();
+      nodes.reset(static_cast<Node*>(p));
+      cap = n;
+      return true;
+    }
+    size_t bytes() const {
+      return cap * sizeof(Node) + frames.capacity() * sizeof(Frame) + names.capacity() * sizeof names[0] +
+             count.capacity() + table.capacity() * sizeof(uint32_t);
+    }
     int16_t one[256];                                      // label of a one-letter symbol, -1: none
   };
   static Work& work() {
     static thread_local Work w;
     return w;
   }
+  // Most bytes of work space that a thread keeps from one net to the next, and
+  // that the process keeps besides, for one large net at a time.  With nothing
+  // kept for it a net of 300 000 nested S takes 7.6 ms, most of it page faults,
+  // instead of 2.8.
+  static constexpr size_t kKept = 2 << 20, kShared = 64 << 20, kLargeText = 64 << 10;
+  struct Large {
+    std::mutex mu;
+    Work work;
+  };
+  static Large& large() {
+    static Large l;
+    return l;
+  }
   Work& W = work();
   const char* p = nullptr;
   const char* end = nullptr;
   size_t n_nodes = 0;
+
+  ~PlainReader() {
+    if (W.bytes() <= kKept) return;
+    if (W.bytes() <= kShared) {
+      std::lock_guard<std::mutex> lock(large().mu);
+      if (large().work.bytes() < W.bytes()) std::swap(large().work, W);
+    }
+    if (W.bytes() > kKept) W = Work();
+  }
 
   static uint8_t cls(char c) { return kChars.of[(unsigned char)c]; }
   char peek() {
@@ -661,7 +701,7 @@ struct PlainReader {
 
   bool term(uint32_t* w_out) {
     W.frames.clear();
-    Node* const nodes = W.nodes.data();
+    Node* nodes = W.nodes.get();
     for (;;) {
       const uint8_t k = cls(peek());
       if (!(k & (kUpper | kLower))) return false;
@@ -679,6 +719,10 @@ struct PlainReader {
         const int lab = len == 1 ? W.one[(unsigned char)*b] : label_of(rules, std::string_view(b, len));
         if (lab < 0) return false;
         arity = rules.arity[(size_t)lab];
+        if (n_nodes == W.cap) {
+          if (n_nodes > kMaxIndex || !W.grow()) return false;
+          nodes = W.nodes.get();
+        }
         me = (uint32_t)n_nodes++;
         Node& nd = nodes[me];
         nd.head = (int32_t)((uint32_t)lab | (net_slot << 8));
@@ -736,8 +780,10 @@ struct PlainReader {
   bool net(const std::string& text) {
     p = text.data();
     end = p + text.size();
-    // an agent takes a letter and, next to another, a bracket or a comma
-    if (W.nodes.size() < text.size() / 2 + 2) W.nodes.resize(text.size() / 2 + 2);
+    if (text.size() >= kLargeText) {
+      std::lock_guard<std::mutex> lock(large().mu);
+      if (large().work.bytes() > W.bytes()) std::swap(large().work, W);
+    }
     W.names.clear();
     W.count.clear();
     memset(W.one, -1, sizeof W.one);
@@ -763,7 +809,7 @@ struct PlainReader {
     }
     if (peek()) return false;
     if ((uint64_t)var_base + out.vars.size() > kMaxIndex || (uint64_t)agent_base + n_nodes > kMaxIndex) return false;
-    out.nodes.assign(W.nodes.begin(), W.nodes.begin() + (ptrdiff_t)n_nodes);
+    out.nodes.assign(W.nodes.get(), W.nodes.get() + n_nodes);
     return true;
   }
 };
