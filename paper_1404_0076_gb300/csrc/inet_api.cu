@@ -621,7 +621,10 @@ inet_status read_nats_device(inet_ctx* ctx, cudaStream_t st, const uint32_t* dro
   const unsigned nb = (m + 255) / 256;
   // every net is walked for kWalkMin round trips; the rest of each longer
   // numeral is ranked on a list of its net's agents only
-  k_nat_walk<<<(m + 7) / 8, 256, 0, st>>>(ctx->dev, droot, m, na, nv, s_label, z_label, kWalkMin, dval, ctl);
+  if (m <= 2u * 64u * (uint32_t)std::max(ctx->num_sms, 1))  // 64 warps an SM
+    k_nat_walk<32><<<(m + 7) / 8, 256, 0, st>>>(ctx->dev, droot, m, na, nv, s_label, z_label, kWalkMin, dval, ctl);
+  else
+    k_nat_walk<4><<<(m + 63) / 64, 256, 0, st>>>(ctx->dev, droot, m, na, nv, s_label, z_label, kWalkMin, dval, ctl);
   CK(cudaGetLastError());
   if (na == 0) return INET_OK;
   if (wait) {

@@ -40,19 +40,25 @@ __device__ __forceinline__ uint32_t jump_slot(uint32_t w, uint32_t n_agents, uin
   return kJumpBad;
 }
 
-// One warp per net: from the interface word, at most `budget` round trips to
-// agents.  Each loads the next 32 slots in the direction the list last went,
+// G lanes per net: from the interface word, at most `budget` round trips to
+// agents.  Each loads the next G slots in the direction the list last went,
 // and goes on as far as the list really leads through them: numerals are
-// mostly laid out in slot order, so a round trip passes up to 32 agents
-// instead of the one that a thread of its own passed (4096 sums of up to 512:
-// readback call 1.12 -> 0.80 ms, most of it now the caller's, the ranking no
-// longer needed).  What bounds it:
-// the round trips of the longest walk, 337 ns each.
+// mostly laid out in slot order, so a round trip passes up to G agents
+// instead of one (4096 sums of up to 512: readback call 1.12 -> 0.80 ms, most
+// of it now the caller's, the ranking no longer needed).  What bounds it: the
+// round trips of the longest walk, 337 ns each, and with several times as many
+// nets as the device holds warps, the waves of walks and what their windows
+// load for nothing.  65 536 Fibonacci numbers, scattered lists: 219 us with 32
+// lanes a net, 103 with 4 (as with one); 16 384 of them 75 and 88, 16 384 sums
+// in slot order 29 and 123.  So 4 lanes where the nets are more than twice the
+// warps that the device holds.
 // out[i] = the numeral, kNatNone, or nat_pending(...) with ctl[0] set.
+template <uint32_t G>
 __global__ void k_nat_walk(Dev d, const uint32_t* roots, uint32_t n, uint32_t n_agents, uint32_t n_vars,
                            int s_label, int z_label, uint32_t budget, unsigned long long* out, uint32_t* ctl) {
-  const uint32_t i = (blockIdx.x * blockDim.x + threadIdx.x) / 32;
-  const int lane = threadIdx.x & 31;
+  const uint32_t i = (blockIdx.x * blockDim.x + threadIdx.x) / G;
+  const uint32_t lane = threadIdx.x % G, base = threadIdx.x % 32 - lane;
+  const unsigned group = (G == 32 ? kFull : (1u << (G & 31)) - 1u) << base;  // the net's lanes of the warp
   if (i >= n) return;
   unsigned long long res = kNatNone;
   uint32_t w = roots[i], k = 0, dir = 1, from = kJumpBad;
@@ -70,15 +76,15 @@ __global__ void k_nat_walk(Dev d, const uint32_t* roots, uint32_t n, uint32_t n_
       break;
     }
     if (from != kJumpBad) dir = e == from - 1 ? ~0u : e == from + 1 ? 1u : dir;
-    const uint32_t at = e + (uint32_t)lane * dir;  // wraps below 0 to a slot out of range
+    const uint32_t at = e + lane * dir;  // wraps below 0 to a slot out of range
     uint2 r = make_uint2(0xFFu, 0u);
     if (at < n_agents) r = __ldcg(reinterpret_cast<const uint2*>(d.node + at));
     const int lab = (int)(r.x & 0xFFu);
     // the agents reached: up to the first that does not lead to its neighbour
-    const unsigned on = __ballot_sync(kFull, lane < 31 && lab == s_label && r.y == mk_agent(at + dir));
+    const unsigned on = __ballot_sync(group, lane < G - 1 && lab == s_label && r.y == mk_agent(at + dir)) >> base;
     const int last = __ffs(~on) - 1;
-    const int lab_last = __shfl_sync(kFull, lab, last);
-    w = __shfl_sync(kFull, r.y, last);
+    const int lab_last = __shfl_sync(group, lab, last, G);
+    w = __shfl_sync(group, r.y, last, G);
     from = e + (uint32_t)last * dir;
     k += (uint32_t)last;
     if (lab_last == z_label) {
