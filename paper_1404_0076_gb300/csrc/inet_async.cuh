@@ -42,30 +42,32 @@
 // fence, exchanges, hand-on; 8 000 to 50 000 cycles) and of the dependent
 // loads inside a run.  The design follows from that: many interactions per
 // turn where a rule allows it, one fence for the whole warp, nothing between
-// lanes but the hand-on.  One interaction per turn, before / runs, now:
-// 2048 Mul nets 10.0 / 4.4 ms, Ackermann(3, 4..8) 66 / 45 ms,
-// Fibonacci(20..25) 133 / 26.6 ms, Fibonacci(22..25) x 64 149 / 41 ms, 512
-// random trees 1.48 / 1.15 ms, a server's 2000 requests 272 / 95 ms.
+// lanes but the hand-on.  With one interaction per turn / now: 2048 Mul nets
+// 9.9 / 4.4 ms, Ackermann(3, 4..8) 66 / 45 ms, Fibonacci(20..25) 81 / 17.4 ms,
+// 16 x Fibonacci(25) 93 / 23 ms, a chain of 20 000 Add 27 / 2.2 ms, 512 trees
+// 1.5 / 1.1 ms, L-System(13) and (22) 0.20 / 0.20 and 0.43 / 0.42 ms.  The
+// figures at the constants below are of the same batches.
 #pragma once
 
 #include "inet_kernels.cuh"
 
 namespace inet {
 
-// 4 freed slots kept per lane: 2048 Mul nets took 12 % longer with 2, 10 % with 8.
 constexpr int kVRes = 8;       // free name slots a lane keeps for itself
-constexpr int kKeep = 4;       // slots of each kind a lane keeps of those it frees; the rest is the warp's
-// Most interactions of one run: of a warp's only lane, of one lane among
-// several, and where most of the warp's lanes reduce rules that do not run
-// (they wait for the run).  Lone: a chain of 20 000 Add 3.4 ms with 64, 2.3
-// with 512.  Among several, 48 / 64 / 96: 2048 Mul nets 5.7 / 5.5 / 6.5 ms,
-// Fibonacci(20..25) 30.6 / 29.5 / 28.5 ms.  Mixed, 16 against 64: 512 random
-// trees within the spread of the runs, and 1.5 against 1.7 ms before runs ended
-// inside (end_run).
+// Slots of each kind a lane keeps of those it frees; the rest is the warp's.
+// 2048 Mul nets 4.5 ms with 2, 4.4 with 4; 4.3 with 8, which holds twice as many
+// back from the others.
+constexpr int kKeep = 4;
+// Interactions after which a run ends (pass_rule looks once a block of 4; a rule
+// that ends the list adds one): of a warp's only lane, of one lane among
+// several, and where most of the warp's lanes reduce rules that do not run and
+// wait for the run.  Lone: the chain 2.2 ms, 3.1 with 64.  Among several, with
+// 32 / 64 / 128: 2048 Mul nets 4.9 / 4.4 / 5.1, Fibonacci 19.8 / 17.4 / 16.6,
+// trees 1.06 / 1.12 / 1.29.  Mixed: trees 1.12 ms, 1.17 with 64.
 constexpr uint32_t kRunLone = 512, kRunMany = 64, kRunMixed = 16;
 constexpr unsigned long long kNoTicket = ~0ull;
 // Slots fetched beyond the need when a warp's stack runs dry (two L2 round
-// trips): L-System(19) 0.29 ms, 0.33 with half as many.
+// trips): L-System(19) 0.30 ms, 0.33 with half as many.
 constexpr uint32_t kFetchA = 64, kFetchV = 32;
 
 // Shared memory of one warp.  kTable: with the value table of the general
@@ -276,21 +278,20 @@ __device__ __noinline__ bool fill_stacks(const Dev& d, WM& W, uint32_t ac, uint3
 }
 
 // Slots for the lanes that lack some for their next interaction (need_a
-// agents, need_v names, 0 for the others; runs: the rule repeats itself along
-// lists), from the warp's stacks into the lanes' columns.  Returns false when
-// the arena is full.  Warp-collective.
+// agents, need_v names, 0 for the others; runs: the rule is reduced in runs;
+// more: what a lane of another rule takes at least), from the warp's stacks into
+// the lanes' columns.  Returns false when the arena is full.  Warp-collective.
 template <class WM>
-__device__ __forceinline__ bool refill(const Dev& d, WM& W, Lane& L, bool runs, uint32_t need_a,
+__device__ __forceinline__ bool refill(const Dev& d, WM& W, Lane& L, bool runs, uint32_t more, uint32_t need_a,
                                        uint32_t need_v, int lane) {
   __syncwarp();
   uint32_t ac = (uint32_t)min(W.an, WM::kAStack), vc = (uint32_t)min(W.vn, WM::kVStack);
-  // what the step needs, and for a run a whole column: a lane of any other
-  // rule may have its last pair here, and what it took for later would send
-  // the next lane to the pools (L-System(19) 0.29 ms, 0.32 with 4 or more)
+  // what the step needs, and for a run a whole column and 4 names (with 2, runs
+  // of Dup and Mul stop for lack of them: 2048 Mul nets 5.5 ms instead of 4.4)
   const uint32_t least_a = (uint32_t)L.na < need_a ? need_a - (uint32_t)L.na : 0u;
   const uint32_t least_v = (uint32_t)L.nv < need_v ? need_v - (uint32_t)L.nv : 0u;
-  uint32_t wa = least_a ? (runs ? (uint32_t)WM::kARes : need_a) - (uint32_t)L.na : 0u;
-  uint32_t wv = least_v ? (runs ? max(need_v, 4u) : need_v) - (uint32_t)L.nv : 0u;
+  uint32_t wa = least_a ? (runs ? (uint32_t)WM::kARes : max(need_a, more)) - (uint32_t)L.na : 0u;
+  uint32_t wv = least_v ? max(need_v, runs ? 4u : more) - (uint32_t)L.nv : 0u;
   uint32_t inc, packed, Ka, Kv;
   // offsets of this lane among the warp's wants
   auto scan = [&]() {
@@ -653,9 +654,8 @@ __device__ __forceinline__ void one_step(const Dev& d, WM& W, Lane& L, int lane,
 // joins each of the run's output streams to something it has at hand, which
 // then goes straight into the open port of the stream's last agent.  That
 // saves a name, the walker's record and a whole step at every list's end, and
-// leaves lists with fewer names in them for whoever walks them next: 512
-// random trees 1.7 -> 1.4 ms, Fibonacci(22..25) x 64 47.5 -> 43.5 ms (and 2048
-// Mul nets 3.9 -> 4.4 ms, whose runs it makes uneven).
+// leaves lists with fewer names in them for whoever walks them next: trees 1.7
+// -> 1.1 ms, Fibonacci 20.0 -> 17.4, 2048 Mul nets 4.8 -> 4.4.
 template <class Rules, int I, int J>
 __host__ __device__ constexpr bool ends_run() {
   constexpr Template R = Rules::kT[I], T = Rules::kT[J];
@@ -936,10 +936,9 @@ __device__ __forceinline__ void run_rule(const Dev& d, WM& W, Lane& L, int lane,
 // owned by this lane, was written before that record was published and does
 // not change.  What bounds it: one L2 round trip (337 ns) per block, partner
 // or name, so a turn of the loop issues whatever each lane waits for at once.
-// A chain of 20 891 Add: 26.2 ms with an interaction at a time, 6.9 ms in
-// run_rule, 2.3 ms here (0.11 us each); 4096 short sums 0.66 -> 0.13 ms.
-// Blocks of 4 against 8 and 16: 2048 Mul nets 4.4 / 5.1 / 5.8 ms,
-// Fibonacci(20..25) 26.6 / 27.3 / 29.5 ms, the chain 2.3 / 2.1 / 1.7 ms.
+// The chain of 20 000 Add takes 0.11 us an interaction (0.34 in run_rule, 1.3
+// with one a turn), 4096 short sums 0.12 ms (0.69).  Blocks of 4 against 8: 2048
+// Mul nets 4.4 / 5.0 ms, the chain 2.2 / 2.0, Fibonacci the same.
 template <bool kTrack, class Rules, int I, class WM>
 __device__ __forceinline__ void pass_rule(const Dev& d, WM& W, Lane& L, int lane, uint32_t a, uint32_t b,
                                           const int4& ra, const int4& rb, uint32_t net, uint32_t lim, Step& S) {
@@ -1075,8 +1074,8 @@ __host__ __device__ constexpr bool walked() {
 // costs nothing where the list is walked as a whole again; where every other
 // rule takes the stream's agents one at a time, each could have had its own as
 // soon as it was made, so such a rule makes one interaction a turn: the
-// L-System's Dup, whose copies only SymA and SymB take (13 steps 0.30 -> 0.18
-// ms, 22 steps 0.60 -> 0.41).  The arithmetic rules' Dup, whose copies Mul and
+// L-System's Dup, whose copies only SymA and SymB take (with the smaller refills,
+// 13 steps 0.30 -> 0.20 ms, 22 steps 0.61 -> 0.42).  The arithmetic rules' Dup, whose copies Mul and
 // Add walk, is the faster in runs: 2048 Mul nets 4.4 ms against 11.5.
 template <class Rules, int I>
 __host__ __device__ constexpr bool runs_along() {
@@ -1222,7 +1221,12 @@ __device__ __forceinline__ void async_interact(const Dev& d, const PackedTpl* tm
   if (lack) {
     bool runs = false;
     if constexpr (Rules::kN > 0) runs = (run_mask<Rules>() >> (ti & 31u)) & 1u;
-    if (!refill(d, W, L, runs, need_a, need_v, lane)) return;  // fatal: the loop stops
+    // In a warp with few pairs a lane may have its last one here, and what it
+    // took for later would send the next lane to the pools (L-System(19) 0.30
+    // ms, 0.32 with 4 or more always); a lane of a busy warp will be back (64
+    // Fibonacci nets 41 ms, 43 with the bare need).
+    const uint32_t more = __popc(__ballot_sync(kFull, valid)) >= 16 ? 4u : 0u;
+    if (!refill(d, W, L, runs, more, need_a, need_v, lane)) return;  // fatal: the loop stops
   }
   // a run keeps the warp's other lanes waiting, and what waits for its output
   uint32_t lim = 1;
@@ -1383,9 +1387,9 @@ __global__ void __launch_bounds__(256, 2) k_async(Dev d) {
   }
   for (uint32_t it = 0;; it++) {
     // stop / slice checks every 4 iterations (on flags loaded during the
-    // iteration before; an iteration may hold a run, and with 16 a slice of
-    // 250 us took 2.2 ms on Fibonacci(22..25) x 64, now 0.56), and when a napping warp's clock says the time
-    // slice is over
+    // iteration before; an iteration may hold a run, and with 16 a slice of 250
+    // us took 2.2 ms on 64 Fibonacci nets instead of 0.56), and when a napping
+    // warp's clock says the time slice is over
     if ((it & 3) == 3 || check_now) {
       if (check_now) {
         if (lane == 1) flag = ld_volatile(&c->astop);

@@ -4,7 +4,7 @@
 // by the rule of that pair, so the specialised kernel applies both as one.
 // One interaction fewer on every path through such a rule, and two agents
 // that are never written: Ackermann(3, 4..8) 68 -> 45 ms together with the
-// runs it makes possible (inet_async.cuh), Fibonacci(22..25) x 64 62 -> 59 ms.
+// runs it makes possible (inet_async.cuh).
 // Plain C++17; no CUDA.
 #pragma once
 

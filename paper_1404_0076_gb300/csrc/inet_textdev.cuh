@@ -227,9 +227,10 @@ __global__ void k_txt_copy_head(const uint32_t* ctl, const TxtElem* b0, const Tx
 // Head, rounds and head's copy of a short list in one launch of one block:
 // block barriers between the rounds instead of two launches each.  What bounds
 // it is the two dependent loads of a round, about 1 us with a few elements a
-// thread, against 5 us for the two launches: reading a word of 89 symbols back takes
-// 0.11 ms instead of 0.18, one of 610 symbols 0.15 instead of 0.22.
-// Beyond kTxtShort elements one block is the slower way (16 a thread and round).
+// thread, against 5 us for the two launches: a word of 377 symbols (3000 elements)
+// is read back in 0.13 ms instead of 0.20, one of 987 (7900) in 0.17 instead of
+// 0.22.  With 12 800 elements both take 0.22 ms, with 20 700 one block takes 0.31
+// and the launches 0.23; kTxtShort is 8 elements a thread and round.
 constexpr uint32_t kTxtShort = 8192;
 __global__ void __launch_bounds__(1024) k_txt_rank_short(Dev d, uint32_t n_c, uint32_t n_agents, uint32_t n_vars,
                                                          const uint32_t* cid, const uint32_t* roots, uint32_t n_el,
