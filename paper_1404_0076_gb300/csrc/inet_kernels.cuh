@@ -368,10 +368,6 @@ __device__ __forceinline__ uint32_t pool_slot(const uint32_t* ring, unsigned lon
   return (uint32_t)(bump_base + (k - ring_avail));
 }
 
-// An equation with a word that is neither an agent nor a name.  Out of line: in
-// the loop over a batch's equations it cost 333 Mul nets 1 % of their time.
-__device__ __noinline__ void report_word(const Dev& d) { set_error(d.ctrl, INET_ERR_STATE, 1); }
-
 // A finished name slot is cleared and staged to be freed.
 template <bool kTrack>
 __device__ __forceinline__ void free_name(const Dev& d, const Smem& s, uint32_t x) {
@@ -651,16 +647,15 @@ __device__ void process_chunk(const Dev& d, const Smem& s, uint32_t base, uint32
       Pair out;
       bool has = false;
       if (k < n_link) {
-        if (is_agent(lt[k]) && is_agent(lu[k])) {
-          out = Pair{idx_of(lt[k]), idx_of(lu[k])};
-          has = true;
-        } else if (lo[k] != kEmpty) {
+        uint32_t t = lt[k];
+        bool on = !is_var(t);  // no exchange was made: two agents, or a word that link_eq reports
+        if (lo[k] != kEmpty) {
           // second arrival: the slot is finished; go on with old = u
-          free_name<kTrack>(d, s, idx_of(lt[k]));
-          has = link_eq<kTrack>(d, s, lo[k], lu[k], &out, 0);
-        } else if (!is_var(lt[k])) {
-          report_word(d);
+          free_name<kTrack>(d, s, idx_of(t));
+          t = lo[k];
+          on = true;
         }
+        if (on) has = link_eq<kTrack>(d, s, t, lu[k], &out, 0);
       }
       push(has, out);
     }
