@@ -92,7 +92,7 @@ def bytes_per_rule(rules: list[dict], batched: bool) -> list[int]:
 # kernel sources they were taken on (sha1 prefix over csrc/inet_kernels.cuh
 # and csrc/inet_async.cuh) and for the kernel they were taken of (the last
 # key: the asynchronous kernel compiled for the rule set, or the general one).
-NCU_TRAFFIC = {("mul2048", "async", "21bd99a5a4f1", True): 6_204_672 + 11_322_624}
+NCU_TRAFFIC = {("mul2048", "async", "cb57e53cd5ce", True): 5_070_336 + 3_860_736}
 
 
 def kernel_source_hash() -> str:
@@ -647,7 +647,8 @@ def main():
                 "jit_state": ji["state"], "jit_compile_ms": round(ji["compile_ms"], 1), "jit_source": ji["source"],
                 "jit_launches": ji["launches"], "jit_msg": ji["msg"],
                 "how": "asynchronous mode compiles k_async for the loaded rule set at its first launch (NVRTC, "
-                       "before the timed steps); warps whose lanes all reduce one rule run that rule's code"}
+                       "before the timed steps); each lane runs its own rule's code, along whole lists where "
+                       "the rule repeats itself"}
     serving = None
     if rank == 0 and world == 1 and not args.no_serving:
         serving = serving_leg(args, local)
