@@ -623,7 +623,7 @@ struct PlainReader {
   // instead of 2.8.
   static constexpr size_t kKept = 2 << 20, kShared = 64 << 20, kLargeText = 64 << 10;
   struct Large {
-    std::mutex mu;
+    std::mutex mu;  // only ever tried: another thread of a process may have held it when this one was forked
     Work work;
   };
   static Large& large() {
@@ -638,8 +638,8 @@ struct PlainReader {
   ~PlainReader() {
     if (W.bytes() <= kKept) return;
     if (W.bytes() <= kShared) {
-      std::lock_guard<std::mutex> lock(large().mu);
-      if (large().work.bytes() < W.bytes()) std::swap(large().work, W);
+      std::unique_lock<std::mutex> lock(large().mu, std::try_to_lock);
+      if (lock && large().work.bytes() < W.bytes()) std::swap(large().work, W);
     }
     if (W.bytes() > kKept) W = Work();
   }
@@ -781,8 +781,8 @@ struct PlainReader {
     p = text.data();
     end = p + text.size();
     if (text.size() >= kLargeText) {
-      std::lock_guard<std::mutex> lock(large().mu);
-      if (large().work.bytes() > W.bytes()) std::swap(large().work, W);
+      std::unique_lock<std::mutex> lock(large().mu, std::try_to_lock);
+      if (lock && large().work.bytes() > W.bytes()) std::swap(large().work, W);
     }
     W.names.clear();
     W.count.clear();
